@@ -301,6 +301,9 @@ int Plan::fill(mg_handle *const *handles, int count)
                 if (!tile_fits(h->lev[l].n, var[k])) var[k] = 0;
         }
         if (flux) var[MG_TILE_PROLONG] = 0;
+        // without post-smoothing the finest level's prolongation also updates the
+        // outer iterate, in the row-tiled kernel (launch_prolong): its blocks
+        if (l == 0 && prm.nu2 == 0) var[MG_TILE_PROLONG] = 0;
         // finest level: one-pass sweep shape of the largest grid if it fits
         // every grid of the table (each with its second iterate buffer)
         int sv = 0;
