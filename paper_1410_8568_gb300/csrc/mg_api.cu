@@ -382,7 +382,6 @@ int Plan::fill(mg_handle *const *handles, int count)
         nst++;
     }
     ot = OuterTable{ov, d_starts + so0, G, starts[nst - 1]};
-    const size_t esz = mixed ? sizeof(float) : sizeof(double);
     tail_smem = 0;
     ntv = 0;
     ncv = 0;
@@ -406,9 +405,8 @@ int Plan::fill(mg_handle *const *handles, int count)
             v.dx[t] = make_fastdiv((unsigned)Lv.n[0]);
             v.dhx[t] = make_fastdiv(Lv.n[0] >= 2 ? (unsigned)(Lv.n[0] >> 1) : 1u);
             v.dy[t] = make_fastdiv((unsigned)Lv.n[1]);
-            v.dq[t] = make_fastdiv(Lv.n[0] >= 4 ? (unsigned)(Lv.n[0] >> 2) : 1u);
             v.a[t] = mixed ? (const void *)Lv.alpha32 : (const void *)Lv.alpha64;
-            off += (flux ? 6 : 5) * (int)Lv.N;
+            off += tail_floats((int)Lv.N, t, v.nt, flux);
             off = (off + 3) & ~3;
         }
         v.x0 = h->lev[lt[g]].x;
@@ -417,7 +415,7 @@ int Plan::fill(mg_handle *const *handles, int count)
         v.st = h->state;
         v.err = h->err + 2;
         v.wait_polls = h->wait_polls;
-        tail_smem = std::max(tail_smem, (size_t)off * esz);
+        tail_smem = std::max(tail_smem, (size_t)off * sizeof(float));
     }
     for (int g = 0; g < G; g++) {
         mg_handle *h = hs[g];
@@ -588,7 +586,7 @@ static void vcycle(Plan &P, Prof &pf, int cyc, bool outer)
     }
     if (P.ntv) {
         pf.begin(s, MG_K_TAIL, 0);
-        launch_tail<T>(P.tv, P.ntv, P.tail_smem, q.omega, q.nu1, q.nu2, cyc, s);
+        launch_tail(P.tv, P.ntv, P.tail_smem, q.omega, q.nu1, q.nu2, cyc, s);
         pf.end(s);
     }
     if (P.ncv) {

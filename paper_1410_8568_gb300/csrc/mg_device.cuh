@@ -266,18 +266,17 @@ struct TailView {
     int nt;                  // tail levels: the first one down to the coarsest
     int per;
     int n[kMaxTail][3];
-    int off[kMaxTail];       // element offset of level t's x, b, wx, wy, wz (N each) in shared memory
-    void *w[kMaxTail][3];    // scaled faces of each tail level (V-cycle precision)
+    int off[kMaxTail];       // element offset of level t's arrays (tail_floats) in shared memory
+    void *w[kMaxTail][3];    // scaled faces of each tail level (FP32)
     void *x0;                // first tail level: correction (out)
     void *b0;                // first tail level: right-hand side (in)
     const double *G;         // coarsest-level inverse
     const GridState *st;
     FastDiv dx[kMaxTail], dhx[kMaxTail], dy[kMaxTail];  // division by n[t][0], n[t][0] / 2, n[t][1]
-    FastDiv dq[kMaxTail];    // division by n[t][0] / 4 (quads per row)
     int *err;                // set to 1 when the staging copies did not complete in time
     long long wait_polls;    // polls of the staging wait before it gives up (kBulkWaitPolls by default)
     int flux;                // flux-conserving prolongation: level t >= 1 also holds its cell
-    const void *a[kMaxTail]; //   coefficients (6th array of the level in shared memory)
+    const void *a[kMaxTail]; //   coefficients
 };
 
 // Blocks of a launch over the cells of an n[0] x n[1] x n[2] level: a block is

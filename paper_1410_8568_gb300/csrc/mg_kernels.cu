@@ -18,7 +18,6 @@
 #include "mg_kernels.h"
 #include "mg_stencil.cuh"
 #include "mg_outer.cuh"
-#include "mg_bulk.cuh"
 
 #include <math.h>
 #include <stdlib.h>
@@ -403,278 +402,6 @@ __global__ void __launch_bounds__(kThreads) k_prolong(const LevelView *__restric
     }
     const int e = find_entry(start, count);
     prolong_entry<T, FLUX, MAYOUT>(lv[e], blockIdx.x - start[e], cyc, ov, false);
-}
-
-// ---------------------------------------------------------------------------
-// The bottom of the V-cycle in one launch: every level of a grid with at most
-// kTailCells cells (and the coarsest solve) is processed by one block of kTailThreads
-// threads, all operands in shared memory, phases separated by block barriers.
-// These levels are too small to fill the GPU; as separate launches they cost
-// a launch latency each (10 per level per cycle) while doing almost no work.
-// The arithmetic is the same as the per-level kernels: red-black half-sweeps
-// (red first, zero initial correction), 8-child restriction of the residual,
-// trilinear prolongation, and the exact coarsest solve e = -G b in FP64.
-// ---------------------------------------------------------------------------
-
-// n elements (n % 4 == 0, both pointers 16-byte aligned) from global to shared memory
-template <class T>
-__device__ __forceinline__ void stage(T *__restrict__ dst, const T *__restrict__ src, int n)
-{
-    if constexpr (sizeof(T) == 4) {
-        for (int c = threadIdx.x; c < (n >> 2); c += blockDim.x)
-            reinterpret_cast<float4 *>(dst)[c] = reinterpret_cast<const float4 *>(src)[c];
-    } else {
-        for (int c = threadIdx.x; c < (n >> 1); c += blockDim.x)
-            reinterpret_cast<double2 *>(dst)[c] = reinterpret_cast<const double2 *>(src)[c];
-    }
-}
-
-template <class T>
-__device__ __forceinline__ T smem_flux(const T *x, const T *wx, const T *wy, const T *wz, int nx,
-                                       int ny, int nz, int per, int i, int j, int k, int c, T xc,
-                                       T &diag)
-{
-    const int sy = nx, sz = nx * ny;
-    T a, d, f;
-    a = wx[c];
-    d = a;
-    f = a * (x[i > 0 ? c - 1 : ((per & 1) ? c + nx - 1 : c)] - xc);
-    if (i + 1 < nx) {
-        a = wx[c + 1];
-        d += a;
-        f += a * (x[c + 1] - xc);
-    } else if (per & 1) {
-        a = wx[c + 1 - nx];
-        d += a;
-        f += a * (x[c + 1 - nx] - xc);
-    }
-    a = wy[c];
-    d += a;
-    f += a * (x[j > 0 ? c - sy : ((per & 2) ? c + sy * (ny - 1) : c)] - xc);
-    if (j + 1 < ny) {
-        a = wy[c + sy];
-        d += a;
-        f += a * (x[c + sy] - xc);
-    } else if (per & 2) {
-        a = wy[c - sy * (ny - 1)];
-        d += a;
-        f += a * (x[c - sy * (ny - 1)] - xc);
-    }
-    a = wz[c];
-    d += a;
-    f += a * (x[k > 0 ? c - sz : ((per & 4) ? c + sz * (nz - 1) : c)] - xc);
-    if (k + 1 < nz) {
-        a = wz[c + sz];
-        d += a;
-        f += a * (x[c + sz] - xc);
-    } else if (per & 4) {
-        a = wz[c - sz * (nz - 1)];
-        d += a;
-        f += a * (x[c - sz * (nz - 1)] - xc);
-    }
-    diag = d;
-    return f;
-}
-
-template <class T>
-__global__ void __launch_bounds__(kTailThreads) k_tail(const TailView *__restrict__ tv, T omega,
-                                                       int nu1, int nu2, int cyc)
-{
-    dep_entry();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *sm = (T *)smem_raw;
-    const TailView &V = tv[blockIdx.x];
-    if (!in_cycle(V.st, cyc)) return;
-    const int nt = V.nt, per = V.per;
-    // stage the faces of every tail level but the coarsest (solved with G) and
-    // the right-hand side of the first by bulk asynchronous copies, issued by
-    // one thread and completed on one mbarrier; levels above the coarsest have
-    // even sizes, so N % 8 == 0: sizes are multiples of 32 bytes and the slab
-    // offsets keep 16-byte alignment
-    __shared__ __align__(8) unsigned long long bar;
-    if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
-        const int N0 = V.n[0][0] * V.n[0][1] * V.n[0][2];
-        unsigned bytes = (unsigned)(N0 * sizeof(T));
-        for (int t = 0; t + 1 < nt; t++) bytes += 3u * (unsigned)(V.n[t][0] * V.n[t][1] * V.n[t][2] * sizeof(T));
-        mbar_arrive_expect_tx(&bar, bytes);
-        for (int t = 0; t + 1 < nt; t++) {
-            const int N = V.n[t][0] * V.n[t][1] * V.n[t][2];
-            T *base = sm + V.off[t];
-            for (int d = 0; d < 3; d++) bulk_g2s(base + (2 + d) * N, V.w[t][d], (unsigned)(N * sizeof(T)), &bar);
-        }
-        bulk_g2s(sm + V.off[0] + N0, V.b0, (unsigned)(N0 * sizeof(T)), &bar);
-    }
-    if (V.flux) {
-        // cell coefficients of the tail's coarse levels (a small odd-sized
-        // coarsest level rules out the vector copy)
-        for (int t = 1; t < nt; t++) {
-            const int N = V.n[t][0] * V.n[t][1] * V.n[t][2];
-            const T *g = (const T *)V.a[t];
-            T *d = sm + V.off[t] + 5 * N;
-            for (int c = threadIdx.x; c < N; c += blockDim.x) d[c] = g[c];
-        }
-    }
-    __syncthreads();  // the barrier is initialised before anyone waits on it
-    // every thread waits (bounded); the outcome is made uniform over the block
-    const int staged = __syncthreads_and(mbar_wait(&bar, 0, V.wait_polls) ? 1 : 0);
-    if (!staged) {
-        // give up on this grid (reported as MG_ETIMEOUT), but let the copies
-        // land before the block's shared memory is released
-        if (threadIdx.x == 0 && V.err) *V.err = 1;
-        mbar_wait(&bar, 0, kBulkWaitPolls);
-        return;
-    }
-
-    // A tail level as a LevelView on shared memory, so that the per-quad
-    // functions of the per-level kernels (half_quad, restrict_pair,
-    // prolong_quad) run here unchanged on levels whose rows are a multiple of 4
-    // cells: one quad per thread at 16^3, 16-byte shared-memory loads, and the
-    // zero-start red half-sweep writes both colours (no clearing pass).  Other
-    // levels take one cell per thread.
-    auto view = [&](int t) {
-        LevelView L;
-        const int N = V.n[t][0] * V.n[t][1] * V.n[t][2];
-        for (int d = 0; d < 3; d++) {
-            L.n[d] = V.n[t][d];
-            L.w[d] = sm + V.off[t] + (2 + d) * N;
-            L.nc[d] = t + 1 < nt ? V.n[t + 1][d] : 1;
-        }
-        L.per = per;
-        L.x = sm + V.off[t];
-        L.b = sm + V.off[t] + N;
-        if (t + 1 < nt) {
-            const int NC = V.n[t + 1][0] * V.n[t + 1][1] * V.n[t + 1][2];
-            L.xc = sm + V.off[t + 1];
-            L.bc = sm + V.off[t + 1] + NC;
-            L.ac = sm + V.off[t + 1] + 5 * NC;
-        }
-        L.zr = 0;
-        return L;
-    };
-
-    // zero: the correction is zero on entry (first red half-sweep of a cycle)
-    auto half = [&](int t, int colour, bool zero) {
-        const int nx = V.n[t][0], ny = V.n[t][1], nz = V.n[t][2], N = nx * ny * nz;
-        T *x = sm + V.off[t];
-        const T *b = x + N, *wx = x + 2 * N, *wy = x + 3 * N, *wz = x + 4 * N;
-        if ((nx & 3) == 0) {
-            const int nq = nx >> 2;
-            for (int q = threadIdx.x; q < (N >> 2); q += blockDim.x) {
-                const int row = fdiv(q, V.dq[t]);
-                const int k = fdiv(row, V.dy[t]);
-                half_quad_sm<T>(x, b, wx, wy, wz, nx, ny, nz, per, row, row - k * ny, k, q - row * nq, colour,
-                                omega, zero);
-            }
-            __syncthreads();
-            return;
-        }
-        if (zero) {
-            // no cell of the level may be read before it is set
-            for (int c = threadIdx.x; c < N; c += blockDim.x) x[c] = T(0);
-            __syncthreads();
-        }
-        const int hx = nx >> 1;
-        for (int m = threadIdx.x; m < (N >> 1); m += blockDim.x) {
-            // m-th cell of the colour: rows of hx cells, the colour's cells at
-            // every other i starting from (colour + j + k) & 1
-            const int row = fdiv(m, V.dhx[t]);
-            const int k = fdiv(row, V.dy[t]);
-            const int j = row - k * ny;
-            const int i = 2 * (m - row * hx) + ((colour + j + k) & 1);
-            const int c = i + nx * row;
-            const T xc = x[c];
-            T d;
-            const T f = smem_flux(x, wx, wy, wz, nx, ny, nz, per, i, j, k, c, xc, d);
-            x[c] = d > T(0) ? xc + omega * relax_div(f - b[c], d) : xc;
-        }
-        __syncthreads();
-    };
-
-    for (int t = 0; t + 1 < nt; t++) {
-        for (int it = 0; it < nu1; it++) {
-            half(t, 0, it == 0);
-            half(t, 1, false);
-        }
-        // restriction of the residual to level t + 1
-        const int nx = V.n[t][0], ny = V.n[t][1], nz = V.n[t][2], N = nx * ny * nz;
-        const int ncx = V.n[t + 1][0], ncy = V.n[t + 1][1], NC = ncx * ncy * V.n[t + 1][2];
-        if ((nx & 3) == 0) {
-            const LevelView L = view(t);
-            const int np = ncx >> 1;
-            for (int g = threadIdx.x; g < (NC >> 1); g += blockDim.x) {
-                const int crow = fdiv(g, V.dq[t]);  // np = nx / 4
-                const int K = fdiv(crow, V.dy[t + 1]);
-                restrict_pair<T>(L, crow, crow - K * ncy, K, g - crow * np, omega);
-            }
-        } else {
-            const T *x = sm + V.off[t];
-            const T *b = x + N, *wx = x + 2 * N, *wy = x + 3 * N, *wz = x + 4 * N;
-            T *bc = sm + V.off[t + 1] + NC;
-            for (int C = threadIdx.x; C < NC; C += blockDim.x) {
-                const int crow = fdiv(C, V.dx[t + 1]);
-                const int K = fdiv(crow, V.dy[t + 1]);
-                const int I = C - crow * ncx, J = crow - K * ncy;
-                T s = T(0);
-                for (int dz = 0; dz < 2; dz++)
-                    for (int dy = 0; dy < 2; dy++)
-                        for (int dx = 0; dx < 2; dx++) {
-                            const int i = 2 * I + dx, j = 2 * J + dy, k = 2 * K + dz;
-                            const int c = i + nx * (j + ny * k);
-                            T d;
-                            s += b[c] - smem_flux(x, wx, wy, wz, nx, ny, nz, per, i, j, k, c, x[c], d);
-                        }
-                bc[C] = s * T(0.125);
-            }
-        }
-        __syncthreads();
-    }
-    {
-        // exact solve on the coarsest level: e = -G b, FP64, one warp per row
-        const int t = nt - 1;
-        const int n = V.n[t][0] * V.n[t][1] * V.n[t][2];
-        T *x = sm + V.off[t];
-        const T *b = x + n;
-        const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-        for (int r = threadIdx.x >> 5; r < n; r += warps) {
-            const double *Gr = V.G + (long long)r * n;
-            double s = 0.0;
-            for (int u = lane; u < n; u += 32) s += Gr[u] * (double)b[u];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) x[r] = (T)(-s);
-        }
-        __syncthreads();
-    }
-    for (int t = nt - 2; t >= 0; t--) {
-        const int nx = V.n[t][0], ny = V.n[t][1], N = nx * ny * V.n[t][2];
-        if ((nx & 3) == 0) {
-            const LevelView L = view(t);
-            const int nq = nx >> 2;
-            for (int q = threadIdx.x; q < (N >> 2); q += blockDim.x) {
-                const int row = fdiv(q, V.dq[t]);
-                const int k = fdiv(row, V.dy[t]);
-                if (V.flux) prolong_quad_flux<T, false>(L, row, row - k * ny, k, q - row * nq, OuterOut{});
-                else prolong_quad<T, false>(L, row, row - k * ny, k, q - row * nq, OuterOut{});
-            }
-        } else {
-            const int nc[3] = {V.n[t + 1][0], V.n[t + 1][1], V.n[t + 1][2]};
-            T *x = sm + V.off[t];
-            const T *ec = sm + V.off[t + 1];
-            const T *ac = ec + 5 * (nc[0] * nc[1] * nc[2]);
-            for (int c = threadIdx.x; c < N; c += blockDim.x) {
-                const int row = fdiv(c, V.dx[t]);
-                const int k = fdiv(row, V.dy[t]);
-                x[c] += V.flux ? prolong_at_flux(ec, ac, nc, per, c - row * nx, row - k * ny, k)
-                               : prolong_at(ec, nc, per, c - row * nx, row - k * ny, k);
-            }
-        }
-        __syncthreads();
-        for (int it = 0; it < nu2; it++) {
-            half(t, 0, false);
-            half(t, 1, false);
-        }
-    }
-    stage((T *)V.x0, sm + V.off[0], V.n[0][0] * V.n[0][1] * V.n[0][2]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1687,17 +1414,6 @@ void launch_prolong_rows(const Table &tb, const OuterView *ov, cudaStream_t s)
     }
 }
 template <class T>
-void launch_tail(const TailView *tv, int count, size_t smem, double omega, int nu1, int nu2, int cyc,
-                 cudaStream_t s)
-{
-    static size_t attr = 0;  // opt in to more than 48 KB of shared memory when needed
-    if (smem > attr) {
-        cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = smem;
-    }
-    launch_k(k_tail<T>, count, kTailThreads, smem, s, tv, (T)omega, nu1, nu2, cyc);
-}
-template <class T>
 void launch_apply(const Table &tb, cudaStream_t s)
 {
     launch_k(k_apply<T>, tb.blocks, kThreads, 0, s, tb.lv, tb.start, tb.count);
@@ -1785,8 +1501,6 @@ template void launch_restrict_rows<float>(const Table &, double, cudaStream_t);
 template void launch_restrict_rows<double>(const Table &, double, cudaStream_t);
 template void launch_prolong_rows<float>(const Table &, const OuterView *, cudaStream_t);
 template void launch_prolong_rows<double>(const Table &, const OuterView *, cudaStream_t);
-template void launch_tail<float>(const TailView *, int, size_t, double, int, int, int, cudaStream_t);
-template void launch_tail<double>(const TailView *, int, size_t, double, int, int, int, cudaStream_t);
 template void launch_apply<float>(const Table &, cudaStream_t);
 template void launch_apply<double>(const Table &, cudaStream_t);
 template void launch_coarse_solve<float>(const CoarseView *, int, int, const OuterView *, cudaStream_t);

@@ -126,8 +126,10 @@ int sweep_blocks(const int n[3], int variant);
 template <class T> void launch_sweep(const Table &, int dir, double omega, int flags, const OuterView *ov,
                                      cudaStream_t);
 // V-cycle stages below the row-tiled levels; cyc as Table::cyc
-template <class T> void launch_tail(const TailView *, int count, size_t smem, double omega, int nu1,
-                                    int nu2, int cyc, cudaStream_t);
+// (the tail: FP32 cycles, mg_tail.cu; tail_floats: shared-memory elements of its
+// level t of nt with N cells)
+int tail_floats(int N, int t, int nt, bool flux);
+void launch_tail(const TailView *, int count, size_t smem, double omega, int nu1, int nu2, int cyc, cudaStream_t);
 template <class T> void launch_apply(const Table &, cudaStream_t);
 template <class T> void launch_coarse_solve(const CoarseView *, int count, int cyc, const OuterView *ov,
                                             cudaStream_t);
