@@ -32,8 +32,8 @@
  * Size rule.  Every axis has n >= 2 cells and the grid fewer than 2^31 cells.
  * All axes are coarsened together while every axis is even and larger than 2.
  * A coarsest grid of at most MG_MAX_COARSE cells is solved exactly (dense
- * inverse); a larger one, up to MG_MAX_COARSE_GMRES cells, by restarted GMRES
- * (Sec. 2.3 item 6).  Every n = m * 2^k with m in {1, 2, 3, 4} has an exact
+ * inverse); a larger one, up to MG_MAX_COARSE_GMRES cells, by GMRES (Sec. 2.3
+ * item 6; the operator is symmetric, so by its short recurrence).  Every n = m * 2^k with m in {1, 2, 3, 4} has an exact
  * coarsest solve (2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256,
  * 384, 512, 768, 1024, ...); sizes with a larger odd factor (e.g. 100 = 25 * 4)
  * take GMRES.
@@ -95,10 +95,10 @@ extern "C" {
 
 #define MG_MAX_COARSE 512 /* most cells of a coarsest grid solved by the dense inverse */
 #define MG_MAX_COARSE_GMRES 32768 /* most cells of any coarsest grid (GMRES above MG_MAX_COARSE) */
-#define MG_GMRES_RESTART 30 /* Krylov vectors per GMRES cycle on the coarsest grid */
+#define MG_GMRES_RESTART 30 /* Krylov vectors a restarted GMRES would keep; the short recurrence keeps 2 */
 
 #define MG_COARSE_AUTO 0  /* coarsest solve: dense inverse up to MG_MAX_COARSE cells, else GMRES */
-#define MG_COARSE_GMRES 1 /* coarsest solve: restarted GMRES whatever the size */
+#define MG_COARSE_GMRES 1 /* coarsest solve: GMRES whatever the size */
 /* outer iteration of the mixed-precision multigrid iteration (mg_params.outer) */
 #define MG_OUTER_FP64 0 /* FP64 residual and FP64 update p += e (Sec. 2.3 with FP32 V-cycles) */
 #define MG_OUTER_XP 1   /* the same steps in extended precision from FP32 arithmetic: p held as a
@@ -147,7 +147,7 @@ typedef struct {
                           level), MG_TILES_ROWS, or a variant 1 .. MG_TILE_VARIANTS - 1 for
                           every level whose rows are a multiple of 4 cells */
     int coarse_solver;     /* MG_COARSE_AUTO (default) or MG_COARSE_GMRES */
-    int coarse_max_iters;  /* GMRES: most Arnoldi steps per coarsest solve (default 300) */
+    int coarse_max_iters;  /* GMRES: most Krylov steps per coarsest solve (default 300) */
     double coarse_tol;     /* GMRES: relative residual of the coarsest solve (default 1e-8); FP64 */
     int adaptive_cycles;   /* 1 (default): after the first refinement step, each step runs as many
                               V-cycles (1 .. inner_cycles) as the last step's measured reduction

@@ -110,7 +110,6 @@ struct Layout {
     size_t xp3[3], xb[2], wlo[3];  // extended-precision outer iteration
     bool xp;
     bool gmres;
-    size_t gm;
     int nblk0;
 };
 
@@ -149,10 +148,9 @@ static int plan_layout(const mg_grid &g, const mg_params &p, Layout &lay)
     }
     const int *nc = lay.n[lay.L - 1];
     const size_t ncells = (size_t)nc[0] * nc[1] * nc[2];
-    // dense inverse for small coarsest grids, GMRES scratch otherwise
+    // dense inverse for small coarsest grids (GMRES keeps its vectors on chip)
     lay.gmres = p.coarse_solver == MG_COARSE_GMRES || ncells > (size_t)kMaxCoarse;
     lay.G = lay.gmres ? 0 : c.take(ncells * ncells * 8);
-    lay.gm = lay.gmres ? c.take((size_t)(kGmresM + 4) * ncells * 8) : 0;
     const size_t N0 = (size_t)g.nx * g.ny * g.nz;
     lay.b0 = c.take(N0 * 8);
     for (int v = 0; v < 4; v++) lay.pcg[v] = p.solver == MG_SOLVER_PCG ? c.take(N0 * 8) : 0;
@@ -437,7 +435,6 @@ int Plan::fill(mg_handle *const *handles, int count)
         v.g = g;
         v.outer = h->L == 1 ? 1 : 0;
         v.gmres = h->gmres ? 1 : 0;
-        v.gm = h->gm;
         v.gm_max = h->prm.coarse_max_iters;
         v.gm_tol = h->prm.coarse_tol;
         if (h->gmres) cv_gmres = true;
@@ -1148,7 +1145,6 @@ int gbmg::handle_alloc(const mg_grid *grid, const mg_params *params, void *strea
     }
     h->gmres = lay.gmres;
     h->G = lay.gmres ? nullptr : (double *)(h->slab + lay.G);
-    h->gm = lay.gmres ? (double *)(h->slab + lay.gm) : nullptr;
     h->b0 = (double *)(h->slab + lay.b0);
     for (int v = 0; v < 4; v++) h->pcg[v] = lay.pcg[v] ? (double *)(h->slab + lay.pcg[v]) : nullptr;
     h->xp = lay.xp;
@@ -1739,7 +1735,6 @@ int mg_coarse_solve(mg_handle *h, int prec, const void *r, void *e)
     v.st = h->dstate;
     v.err = h->err + 1;
     v.gmres = h->gmres ? 1 : 0;
-    v.gm = h->gm;
     v.gm_max = h->prm.coarse_max_iters;
     v.gm_tol = h->prm.coarse_tol;
     CK(cudaMemcpyAsync(h->dcview, &v, sizeof(v), cudaMemcpyHostToDevice, h->stream));

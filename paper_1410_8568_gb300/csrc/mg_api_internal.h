@@ -93,7 +93,6 @@ struct mg_handle {
     signed char tile[4][MG_MAX_LEVELS] = {};  // launch shape per kernel (MG_TILE_*) and level
     double *pcg[4] = {nullptr, nullptr, nullptr, nullptr};  // CG: r, z, d, q (FP64, finest level)
     bool gmres = false;        // coarsest grid solved by GMRES (no dense inverse)
-    double *gm = nullptr;      // GMRES scratch
     // extended-precision outer iteration (mixed precision, multigrid iteration):
     // three-float iterate, float-pair right-hand side, low parts of the level-0 faces
     bool xp = false;

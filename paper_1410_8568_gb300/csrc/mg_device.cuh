@@ -21,7 +21,6 @@ constexpr int kSeg = 64;          // x extent of a warp's row segment (2 cells p
 constexpr int kCSeg = 32;         // x extent of a warp's coarse row segment (restriction)
 constexpr int kMaxCoarse = 512;   // most cells of the coarsest grid (dense inverse)
 constexpr int kMaxCoarseGmres = 32768;  // most cells of a coarsest grid solved by GMRES
-constexpr int kGmresM = 30;       // Krylov vectors per GMRES cycle
 constexpr int kPart = 4;          // doubles of reduction partials per block
 constexpr int kOuterCap = 608;    // most blocks of one grid in an outer (FP64) launch: 4 per SM
 
@@ -250,9 +249,8 @@ struct CoarseView {
     int *err;            // set-up error flag (non-positive pivot)
     int g;               // index of the grid in its plan
     int outer;           // 1 if this is also the finest level (p += e happens here)
-    int gmres;           // 1: solved by restarted GMRES (G unused)
-    double *gm;          // GMRES scratch: b, e, w, then kGmresM + 1 Krylov vectors (FP64, nc each)
-    int gm_max;          // most Arnoldi steps
+    int gmres;           // 1: solved by GMRES (G unused)
+    int gm_max;          // most Krylov steps
     double gm_tol;       // relative residual
 };
 
