@@ -114,11 +114,11 @@ def read_peaks():
 
 def kernel_source_hash():
     """Hash of the sources that define the profiled smoother kernels: the flat
-    half-sweep (mg_tiles.cu), the one-pass sweeps (mg_fused.cu, mg_staged.cu), the per-quad
+    half-sweep (mg_tiles.cu), the one-pass sweeps (mg_fused.cu, mg_march.cu), the per-quad
     relaxation they share (mg_stencil.cuh, mg_xprec.cuh) and the views and
     launch helpers (mg_device.cuh, mg_launch.cuh)."""
     h = hashlib.sha256()
-    for f in ("mg_tiles.cu", "mg_fused.cu", "mg_staged.cu", "mg_stencil.cuh", "mg_xprec.cuh", "mg_device.cuh",
+    for f in ("mg_tiles.cu", "mg_fused.cu", "mg_march.cu", "mg_stencil.cuh", "mg_xprec.cuh", "mg_device.cuh",
               "mg_launch.cuh"):
         with open(os.path.join(ROOT, "paper_1410_8568_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
@@ -218,12 +218,11 @@ def level_shapes(shape):
 
 
 def count_launches(shape, iters, steps, nu1=2, nu2=2, inner=3, tail_cells=4096, mixed=True, pcg=False,
-                   xp=False, onepass=False, staged=False):
+                   xp=False, onepass=()):
     """Kernels of one solve step: coefficient set-up, prologue, refinement (or CG) steps, epilogue.
     In FP32 cycles the levels of at most tail_cells cells (below the finest) run in one launch;
     with more than one V-cycle per refinement step each step starts with a step-control kernel.
-    onepass: the finest level runs one launch per red-black sweep instead of two; staged: with a
-    staged shape, the post-sweeps of a step's last cycle still run as half-sweep pairs."""
+    onepass: the levels (by index) that run one launch per red-black sweep instead of two."""
     lv = level_shapes(shape)
     L = len(lv)
     lt = next((l for l in range(1, L - 1) if math.prod(lv[l]) <= tail_cells), L) if mixed else L
@@ -241,9 +240,10 @@ def count_launches(shape, iters, steps, nu1=2, nu2=2, inner=3, tail_cells=4096, 
     else:
         per_step = 3 + (1 if inner > 1 else 0)  # residual, finalize, loop control (+ step control)
     epilogue = 3                       # sum p, mean, p - mean
-    if onepass and not pcg:
-        cycle -= nu1 + nu2
-        per_step += nu2 if staged else 0
+    # (below the finest level the first red half-sweep was not a launch of its own)
+    for l in onepass if not pcg else ():
+        if l < normal:
+            cycle -= nu1 + nu2 - (1 if l > 0 else 0)
     return setup + prologue + iters * cycle + steps * per_step + epilogue
 
 
@@ -788,6 +788,9 @@ def run_single(args, rank, world, local_rank, dist):
             b = ALG_BPC[name] * N
             per_kernel[name] = {"avg_launch_us": us, "algorithmic_bytes_per_launch": b,
                                 "achieved_gbs": b / (us * 1e3), "frac": b / (us * 1e3) / peak, "bound": "hbm"}
+    # levels whose sweeps were one launch each: nu1 + nu2 smoothing launches per prolongation
+    onepass = [l for l in range(S.num_levels())
+               if 0 < S.profile_read(gbmg.K_SMOOTH, l)[0] == 4 * S.profile_read(gbmg.K_PROLONG, l)[0]]
     S.profile(False)
     fp64_rate = gbmg.probe_fp64_rate(stream=stream)
     res_us = 1000.0 * ms_r / max(1, n_r)
@@ -834,8 +837,7 @@ def run_single(args, rank, world, local_rank, dist):
     if rank == 0:
         m, f = results["mixed"], results["fp64"]
         launches = args.steps * count_launches(P.shape, m["iters"], m["refine_steps"], inner=m["inner"],
-                                               pcg=args.solver == "pcg", onepass=sv > 0,
-                                               staged=sv > 0 and gbmg.sweep_shape(sv)[2] > 0)
+                                               pcg=args.solver == "pcg", onepass=onepass)
         xp = results.get("mixed_xp")
         line = {
             "metric": METRIC, "value": m["value"], "unit": "solves/s", "n_gpus": world,

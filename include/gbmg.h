@@ -154,14 +154,15 @@ typedef struct {
                               rate predicts the tolerance needs, with a 10% margin on the rate;
                               0: always inner_cycles.  Either way a solve stops at max_iters cycles */
     int outer;             /* MG_OUTER_FP64 (default) or MG_OUTER_XP */
-    int sweep;             /* finest-level red-black sweep: MG_SWEEP_AUTO (default: the faster of
-                              two half-sweep launches per sweep and the one-pass sweep shapes that
-                              fit, timed at create), MG_SWEEP_HALF, or a one-pass shape
-                              1 .. MG_SWEEP_VARIANTS - 1 (used where it fits, else MG_SWEEP_HALF).
-                              The one-pass sweep needs even nu1 and nu2 and a second iterate buffer
-                              on the finest level (4 B per cell mixed, 8 B FP64); the staged shapes
-                              (tile_x of mg_sweep_shape nonzero) run in FP32 cycles only.  Every
-                              choice gives bitwise the same result */
+    int sweep;             /* red-black sweeps: MG_SWEEP_AUTO (default: in FP32 cycles the marching
+                              one-pass sweep on every level where a rule on its size finds it the
+                              faster, else the half-sweep pair or a whole-row shape, timed at
+                              create), MG_SWEEP_HALF, or a one-pass shape 1 .. MG_SWEEP_VARIANTS - 1
+                              on the finest level (used where it fits, else MG_SWEEP_HALF).  The
+                              one-pass sweep needs even nu1 and nu2 and a second iterate buffer on
+                              its level (4 B per cell mixed, 8 B FP64); the tiled shapes (tile_x of
+                              mg_sweep_shape nonzero) run in FP32 cycles only.  Every choice gives
+                              bitwise the same result */
 } mg_params;
 
 typedef struct {
@@ -365,7 +366,7 @@ int mg_restrict_residual(mg_handle *h, int level, int prec, const void *b, const
  * choice on that level.  MG_EINVAL if the shape does not fit the level: an
  * even number of cells along a periodic y or z axis, and for a whole-row shape
  * rows of a multiple of 4 cells, at most a third of the shape's threads quads
- * per row; for a staged shape rows of a multiple of its tile_x cells and
+ * per row; for a tiled shape rows of a multiple of its tile_x cells and
  * prec = MG_PREC_MIXED. */
 int mg_smooth_onepass(mg_handle *h, int level, int prec, const void *b, void *x, void *work, int sweeps,
                       int variant);
@@ -488,10 +489,12 @@ int mg_tile_shape(int variant, int *threads, int *items_per_thread);
  * block owns a strip of full rows (as many as the threads allow at one thread
  * per 4-cell quad, less the two halo rows whose red cells it recomputes) of a
  * chunk of planes, and reads its operands from global memory.  tile_x > 0
- * (staged shapes, FP32 cycles): a block owns a tile of tile_x cells along x
- * and up to 14 rows of a chunk of planes, and copies each plane of its
- * operands (with the halo cells it recomputes) into shared memory two planes
- * ahead of the relaxation. */
+ * (FP32 cycles): a block owns a tile of tile_x cells along x and up to 14 rows
+ * of a chunk of planes and marches up it with its operands copied into shared
+ * memory three planes ahead (16 row warps; the threads reported count one warp
+ * more, for the halo cells, whose work the row warps share).  A handle that
+ * chose the marching sweep by its rule reports the first tiled shape whose
+ * planes hold its chunk, also for rows that are not whole tiles. */
 int mg_sweep_shape(int variant, int *threads, int *planes, int *tile_x);
 
 /* Forget every cached choice (the next mg_create times again). */

@@ -102,7 +102,7 @@ struct Layout {
     int L;
     int n[MG_MAX_LEVELS][3];
     size_t w64[MG_MAX_LEVELS][3], w32[MG_MAX_LEVELS][3], x[MG_MAX_LEVELS], b[MG_MAX_LEVELS];
-    size_t x2;  // second iterate buffer of the finest level (one-pass sweep), 0 if none
+    size_t x2[MG_MAX_LEVELS];  // second iterate buffer (one-pass sweep), 0 if none
     size_t dinv[MG_MAX_LEVELS];  // FP64 cycles: inverse diagonals of the relaxed levels (0 if none)
     size_t alpha64[MG_MAX_LEVELS], alpha32[MG_MAX_LEVELS];
     size_t G, b0, part, err, state, dstate, dview, dstart, dcview, setup_cv, total;
@@ -113,14 +113,18 @@ struct Layout {
     int nblk0;
 };
 
-// the finest level can run one-pass sweeps (mg_fused.cu): even nu1 and nu2
-// (the sweeps alternate between two buffers and must end in the first) and
-// some one-pass shape fits it
-static bool onepass_possible(const mg_grid &g, const mg_params &p, const int n[3])
+// a level can run one-pass sweeps: even nu1 and nu2 (the sweeps alternate
+// between two buffers and must end in the first) and, on the finest level, some
+// one-pass shape fits it; below it, the marching sweep is the faster one
+// (march_chunk; FP32 cycles with the sweep left to the library)
+static bool onepass_possible(const mg_grid &g, const mg_params &p, const int n[3], int level)
 {
     if (p.sweep == MG_SWEEP_HALF || (p.nu1 & 1) || (p.nu2 & 1)) return false;
     const int per = (g.bc[0] == MG_BC_PERIODIC ? 1 : 0) | (g.bc[1] == MG_BC_PERIODIC ? 2 : 0) |
                     (g.bc[2] == MG_BC_PERIODIC ? 4 : 0);
+    if (level > 0)
+        return p.sweep == MG_SWEEP_AUTO && p.precision == MG_PREC_MIXED && march_chunk(n, per) > 0;
+    if (p.precision == MG_PREC_MIXED && p.sweep == MG_SWEEP_AUTO && march_chunk(n, per) > 0) return true;
     for (int v = 1; v < kSweepVariants; v++)
         if (sweep_fits(n, per, v, p.precision == MG_PREC_MIXED)) return true;
     return false;
@@ -139,7 +143,7 @@ static int plan_layout(const mg_grid &g, const mg_params &p, Layout &lay)
         for (int d = 0; d < 3; d++) lay.w32[l][d] = mixed ? c.take(N * 4) : 0;
         lay.x[l] = c.take(N * vs);
         lay.b[l] = c.take(N * vs);
-        if (l == 0) lay.x2 = (lay.L > 1 && onepass_possible(g, p, lay.n[0])) ? c.take(N * vs) : 0;
+        lay.x2[l] = (l + 1 < lay.L && onepass_possible(g, p, lay.n[l], l)) ? c.take(N * vs) : 0;
         // FP64 cycles relax every level but the coarsest with its inverse diagonal
         lay.dinv[l] = (!mixed && l + 1 < lay.L) ? c.take(N * 8) : 0;
         const bool flux = l > 0 && p.prolongation == MG_PROLONG_FLUX;
@@ -213,7 +217,7 @@ int Plan::alloc(int cap)
 {
     capacity = cap;
     const int LV = cap * (MG_MAX_LEVELS - 1);
-    const int ST = 3 * (cap + 1) * (MG_MAX_LEVELS - 1) + 2 * (cap + 1);
+    const int ST = 4 * (cap + 1) * (MG_MAX_LEVELS - 1) + (cap + 1);
     Carve c;
     o_lv = c.take((size_t)LV * sizeof(LevelView));
     o_starts = c.take((size_t)ST * sizeof(int));
@@ -276,8 +280,35 @@ int Plan::fill(mg_handle *const *handles, int count)
         down[l] = Table{d_lv, d_starts, 0, 0};
         rest[l] = down[l];
         half[l] = down[l];
+        sweep[l] = down[l];
     }
-    sweep0 = Table{d_lv, d_starts, 0, 0};
+    // one-pass sweep shape of level l's table: 0 for half-sweeps, a whole-row shape
+    // (finest level), kMarchVariant for the marching sweep
+    auto table_sweep = [&](int l, const std::vector<int> &lt) {
+        int sv = 0;
+        long long big = -1;
+        for (int g = 0; g < G; g++) {
+            mg_handle *h = hs[g];
+            if (l + 1 >= h->L || l >= lt[g] || h->lev[l].N <= big) continue;
+            big = h->lev[l].N;
+            sv = h->mkc[l] ? kMarchVariant : l == 0 ? h->tile[MG_TILE_SWEEP][0] : 0;
+        }
+        for (int g = 0; g < G && sv > 0; g++) {
+            mg_handle *h = hs[g];
+            if (l + 1 >= h->L || l >= lt[g]) continue;
+            if (!h->lev[l].x2 || !(sv == kMarchVariant ? h->mixed && march_fits(h->lev[l].n, h->per)
+                                                       : sweep_fits(h->lev[l].n, h->per, sv, h->mixed)))
+                sv = 0;
+        }
+        return sv;
+    };
+    // planes per block of a grid's marching sweep: its own chunk alone; among
+    // others, whose blocks fill the SMs too, at least 16 (a block of kc planes
+    // relaxes the red cells of kc + 2)
+    auto table_chunk = [&](const mg_handle *h, int l) {
+        const int kc = h->mkc[l] ? h->mkc[l] : 16;
+        return G == 1 ? kc : std::max(kc, 16);
+    };
     for (int l = 0; l + 1 < Lmax; l++) {
         const int lv0 = nlv;
         int sf0 = nst, sc0, sh0, cnt = 0;
@@ -302,24 +333,11 @@ int Plan::fill(mg_handle *const *handles, int count)
         // without post-smoothing the finest level's prolongation also updates the
         // outer iterate, in the row-tiled kernel (launch_prolong): its blocks
         if (l == 0 && prm.nu2 == 0) var[MG_TILE_PROLONG] = 0;
-        // finest level: one-pass sweep shape of the largest grid if it fits
-        // every grid of the table (each with its second iterate buffer)
-        int sv = 0;
-        if (l == 0) {
-            long long big = -1;
-            for (int g = 0; g < G; g++) {
-                mg_handle *h = hs[g];
-                if (l + 1 >= h->L || l >= lt[g] || h->lev[0].N <= big) continue;
-                big = h->lev[0].N;
-                sv = h->tile[MG_TILE_SWEEP][0];
-            }
-            for (int g = 0; g < G && sv > 0; g++) {
-                mg_handle *h = hs[g];
-                if (l + 1 >= h->L || l >= lt[g]) continue;
-                if (!h->lev[0].x2 || !sweep_fits(h->lev[0].n, h->per, sv, h->mixed)) sv = 0;
-            }
-        }
-        // three prefix arrays (four on the finest level), each count + 1 long,
+        // one-pass sweep of the largest grid if it fits every grid of the table
+        // (each with its second iterate buffer): the marching sweep, or on the
+        // finest level a whole-row shape
+        const int sv = table_sweep(l, lt);
+        // three prefix arrays (four with one-pass sweeps), each count + 1 long,
         // laid out one after the other
         std::vector<int> sf{0}, sc{0}, sh{0}, sw{0};
         for (int g = 0; g < G; g++) {
@@ -342,14 +360,16 @@ int Plan::fill(mg_handle *const *handles, int count)
             v.st = h->state;
             v.ac = mixed ? (const void *)C.alpha32 : (const void *)C.alpha64;
             // the next level has its own half-sweeps (neither a tail level nor
-            // the coarsest): its zero-start red half-sweep rides on this restriction
-            v.zr = (l + 1 < lt[g] && l + 2 < h->L) ? 1 : 0;
+            // the coarsest, and no one-pass sweeps): its zero-start red half-sweep
+            // rides on this restriction
+            v.zr = (l + 1 < lt[g] && l + 2 < h->L && table_sweep(l + 1, lt) == 0) ? 1 : 0;
             for (int d = 0; d < 3; d++) v.wc[d] = mixed ? (const void *)C.w32[d] : (const void *)C.w64[d];
             fill_fastdiv(v);
             v.x2 = F.x2;
             v.dinv = mixed ? nullptr : F.dinv;
             v.dinvc = mixed ? nullptr : C.dinv;
-            if (sv > 0) sw.push_back(sw.back() + sweep_layout(v, sv));
+            if (sv > 0)
+                sw.push_back(sw.back() + (sv >= kMarchVariant ? march_layout(v, table_chunk(h, l)) : sweep_layout(v, sv)));
             sf.push_back(sf.back() + prolong_blocks_v(F.n, C.n, var[MG_TILE_PROLONG]));
             sc.push_back(sc.back() + restrict_blocks_v(F.n, C.n, var[MG_TILE_RESTRICT]));
             sh.push_back(sh.back() + half_sweep_blocks_v(F.n, var[MG_TILE_HALF]));
@@ -366,12 +386,12 @@ int Plan::fill(mg_handle *const *handles, int count)
         if (sv > 0) {
             const int sw0 = nst;
             for (int v : sw) starts[nst++] = v;
-            sweep0 = Table{d_lv + lv0, d_starts + sw0, cnt, sw.back(), sv};
+            sweep[l] = Table{d_lv + lv0, d_starts + sw0, cnt, sw.back(), sv};
         }
         // a one-grid table also hands its view to the kernels by value (the
         // host copy stays in the staging buffer, rewritten only by fill)
         if (cnt == 1) down[l].hv = rest[l].hv = half[l].hv = lv + lv0;
-        if (cnt == 1 && sv > 0) sweep0.hv = lv + lv0;
+        if (cnt == 1 && sv > 0) sweep[l].hv = lv + lv0;
     }
     const int so0 = nst;
     starts[nst++] = 0;
@@ -555,17 +575,17 @@ static void vcycle(Plan &P, Prof &pf, int cyc, bool outer)
         const Table H = at(P.half[l]);
         if (H.count == 0) continue;
         const bool zero = !(l == 0 && cyc > 0);
-        if (l == 0 && P.sweep0.count > 0) {
+        if (P.sweep[l].count > 0) {
             // one-pass sweeps, alternating between the two iterate buffers
             // (nu1 even: the last one writes x)
-            const Table W = at(P.sweep0);
+            const Table W = at(P.sweep[l]);
             for (int it = 0; it < q.nu1; it++) {
                 pf.begin(s, MG_K_SMOOTH, l);
                 launch_sweep<T>(W, it & 1, q.omega, (it == 0 && zero) ? kHalfZero : 0, nullptr, s);
                 pf.end(s);
             }
         }
-        for (int it = 0; it < q.nu1 && !(l == 0 && P.sweep0.count > 0); it++) {
+        for (int it = 0; it < q.nu1 && P.sweep[l].count == 0; it++) {
             // below the finest level the restriction into this level already
             // did the zero-start red half-sweep of every grid in this table
             if (!(it == 0 && l > 0)) {
@@ -599,12 +619,10 @@ static void vcycle(Plan &P, Prof &pf, int cyc, bool outer)
         pf.begin(s, MG_K_PROLONG, l);
         launch_prolong<T>(at(P.down[l]), (top && q.nu2 == 0) ? P.ov : nullptr, s);
         pf.end(s);
-        // the post-sweeps that end a refinement step also add the final values
-        // to the outer iterate: as half-sweep launches where the one-pass shape
-        // is a staged one (bitwise the same; the staged kernel's instance with
-        // that update runs out of registers and takes twice as long)
-        if (l == 0 && P.sweep0.count > 0 && !(top && sweep_shape(P.sweep0.variant).tile_x)) {
-            const Table W = at(P.sweep0);
+        // the last post-sweep of a refinement step also adds the final values to
+        // the outer iterate
+        if (P.sweep[l].count > 0) {
+            const Table W = at(P.sweep[l]);
             for (int it = 0; it < q.nu2; it++) {
                 // the last sweep adds both colours' final values
                 const int fl = (top && it == q.nu2 - 1) ? kHalfOuter : 0;
@@ -1137,7 +1155,7 @@ int gbmg::handle_alloc(const mg_grid *grid, const mg_params *params, void *strea
         }
         L.N = (long long)L.n[0] * L.n[1] * L.n[2];
         L.x = h->slab + lay.x[l];
-        L.x2 = (l == 0 && lay.x2) ? (void *)(h->slab + lay.x2) : nullptr;
+        L.x2 = lay.x2[l] ? (void *)(h->slab + lay.x2[l]) : nullptr;
         L.dinv = lay.dinv[l] ? (double *)(h->slab + lay.dinv[l]) : nullptr;
         L.alpha64 = lay.alpha64[l] ? (double *)(h->slab + lay.alpha64[l]) : nullptr;
         L.alpha32 = lay.alpha32[l] ? (float *)(h->slab + lay.alpha32[l]) : nullptr;
@@ -1657,9 +1675,12 @@ int mg_smooth_onepass(mg_handle *h, int level, int prec, const void *b, void *x,
     if (variant < 0 || variant >= kSweepVariants) return MG_EINVAL;
     if (prec != MG_PREC_FP64 && prec != MG_PREC_MIXED) return MG_EINVAL;
     if (prec == MG_PREC_MIXED && !h->mixed) return MG_EINVAL;
-    if (variant == 0) variant = level == 0 ? h->tile[MG_TILE_SWEEP][0] : 0;
     const HLevel &L = h->lev[level];
-    if (!sweep_fits(L.n, h->per, variant, prec == MG_PREC_MIXED)) return MG_EINVAL;
+    // the handle's choice on the finest level (a marching sweep by its own chunk)
+    const bool own = variant == 0 && level == 0;
+    if (own) variant = h->tile[MG_TILE_SWEEP][0];
+    const int kc = own && prec == MG_PREC_MIXED ? h->mkc[0] : 0;
+    if (!kc && !sweep_fits(L.n, h->per, variant, prec == MG_PREC_MIXED)) return MG_EINVAL;
     LevelView v;
     memset(&v, 0, sizeof(v));
     for (int d = 0; d < 3; d++) {
@@ -1673,7 +1694,7 @@ int mg_smooth_onepass(mg_handle *h, int level, int prec, const void *b, void *x,
     v.st = h->dstate;
     v.dinv = prec == MG_PREC_FP64 ? L.dinv : nullptr;
     fill_fastdiv(v);
-    const int blocks = sweep_layout(v, variant);
+    const int blocks = kc ? march_layout(v, kc) : sweep_layout(v, variant);
     const int starts[2] = {0, blocks};
     CK(cudaMemcpyAsync(h->dview, &v, sizeof(v), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemcpyAsync(h->dstart, starts, sizeof(starts), cudaMemcpyHostToDevice, h->stream));

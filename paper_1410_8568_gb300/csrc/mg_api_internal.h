@@ -33,7 +33,7 @@ struct HLevel {
     double *w64[3];  // alpha / h^2, FP64
     float *w32[3];   // FP32 copy (mixed precision only)
     void *x;         // V-cycle iterate / correction (V-cycle precision)
-    void *x2;        // finest level: second iterate buffer of the one-pass sweep (or null)
+    void *x2;        // second iterate buffer of the one-pass sweep (or null)
     void *b;         // V-cycle right-hand side (V-cycle precision)
     double *dinv;    // FP64 cycles: inverse diagonal 1 / (sum of the cell's faces), levels below the coarsest
     double *alpha64; // cell coefficients (flux-conserving prolongation, levels >= 1), FP64
@@ -91,6 +91,7 @@ struct mg_handle {
     cudaStream_t io_stream = nullptr;  // host-call input copies that overlap the face set-up
     cudaEvent_t io_ready = nullptr;
     signed char tile[4][MG_MAX_LEVELS] = {};  // launch shape per kernel (MG_TILE_*) and level
+    int mkc[MG_MAX_LEVELS] = {};              // planes per block of the level's marching sweep (0: none)
     double *pcg[4] = {nullptr, nullptr, nullptr, nullptr};  // CG: r, z, d, q (FP64, finest level)
     bool gmres = false;        // coarsest grid solved by GMRES (no dense inverse)
     // extended-precision outer iteration (mixed precision, multigrid iteration):
@@ -123,7 +124,7 @@ struct Plan {
     Table down[MG_MAX_LEVELS];  // prolongation (fine tiles of level l)
     Table rest[MG_MAX_LEVELS];  // restriction (coarse tiles of level l+1)
     Table half[MG_MAX_LEVELS];  // red-black half-sweeps of level l
-    Table sweep0;               // one-pass sweeps of the finest level (count 0: half-sweeps)
+    Table sweep[MG_MAX_LEVELS]; // one-pass sweeps of level l (count 0: half-sweeps)
     CoarseView *cv = nullptr;   // coarsest solves of the grids without a tail
     int ncv = 0;
     bool cv_dense = false, cv_gmres = false;  // which coarse kernels the cv table needs

@@ -126,9 +126,10 @@ __host__ __device__ constexpr TileShape tile_shape(int v)
 // Launch shapes of the one-pass red-black sweep: B threads per block and Kc
 // planes per block (a chunk of the z march).  Variants 1 .. 6 (mg_fused.cu):
 // a block owns a strip of full rows, a thread per quad of each row of the
-// strip (2 halo rows included).  Variants 7 .. 10 (mg_staged.cu, FP32 cycles):
-// a block owns a tile of tile_x = 128 cells of up to 14 rows and stages its
-// operands in shared memory.  Variant 0 is no one-pass sweep (two half-sweep
+// strip (2 halo rows included).  Variants 7 .. 10 (mg_march.cu, FP32 cycles): a
+// block of 16 row warps (B counts one more, for the halo cells' share) owns a
+// tile of tile_x = 128 cells of up to 14 rows and marches with its operands
+// staged in shared memory.  Variant 0 is no one-pass sweep (two half-sweep
 // launches per sweep).
 constexpr int kSweepVariants = 11;
 struct SweepShape {
@@ -174,11 +175,12 @@ struct LevelView {
     // half-sweep, from the restricted right-hand side and that level's faces wc
     int zr;
     const void *wc[3];
-    // one-pass red-black sweep (finest level): the second iterate buffer (a
+    // one-pass red-black sweep: the second iterate buffer (a
     // sweep reads one and writes the other), rows per strip, planes per chunk,
     // strips per plane, and division by the strips and by the quads per row
     void *x2;
     int fR, fKc, fS;
+    int fT;  // marching sweep: quads of a tile along x
     FastDiv dfS, dfq;
     // FP64 cycles: inverse diagonals (1 / sum of the cell's face coefficients,
     // 0 for a cell without faces) of this level and of the next coarser one;

@@ -296,7 +296,7 @@ bool sweep_fits(const int n[3], int per, int v, bool fp32)
 int sweep_layout(LevelView &v, int variant)
 {
     const SweepShape sh = sweep_shape(variant);
-    if (sh.tile_x) return staged_layout(v, sh.Kc);
+    if (sh.tile_x) return march_layout(v, sh.Kc);
     const int nq = v.n[0] >> 2, ny = v.n[1], nz = v.n[2];
     const int rmax = sh.B / nq - 2;
     const int strips = (ny + rmax - 1) / rmax;
@@ -320,12 +320,12 @@ template <class T>
 void launch_sweep(const Table &tb, int dir, double omega, int flags, const OuterView *ov, cudaStream_t s)
 {
     if (tb.blocks == 0) return;
-    const SweepShape sh = sweep_shape(tb.variant);
-    if (sh.tile_x) {
-        // FP32 only: sweep_fits() offers the staged shapes to FP32 cycles alone
-        if constexpr (sizeof(T) == 4) launch_sweep_staged(tb, dir, omega, flags, ov, s);
+    if (tb.variant >= kMarchVariant) {
+        // FP32 only: sweep_fits() offers these shapes to FP32 cycles alone
+        if constexpr (sizeof(T) == 4) launch_march(tb, dir, omega, flags, ov, s);
         return;
     }
+    const SweepShape sh = sweep_shape(tb.variant);
     const bool mo = (flags & kOuter) != 0;
     if (sh.B == 1024) {
         if (mo) launch_sweep_b<T, 1024, true>(tb, dir, omega, flags, ov, s);

@@ -119,8 +119,8 @@ struct LoadPlain {
 // the row length is a multiple of 4 a thread owns an aligned quad of 4 cells of
 // a row (one 16-byte vector per operand for FP32, two for FP64), relaxes the 2
 // cells of the launch's colour and writes the other two back unchanged;
-// otherwise (small coarse levels) one cell per thread.  The FP32 cycle uses the
-// 2-ulp division (__fdividef): the inner cycle is a preconditioner and only
+// otherwise (small coarse levels) one cell per thread.  The FP32 cycle uses a
+// 2-ulp division (relax_div): the inner cycle is a preconditioner and only
 // steers convergence; the FP64 path divides exactly.
 //
 // flags: kZeroGuess  (red launch) the iterate is zero on entry: red cells get
@@ -165,14 +165,14 @@ __device__ __forceinline__ void half_body(const LevelView &L, int lb, int colour
                     v = di[c] > T(0) ? omega * ((-b[c]) * di[c]) : T(0);
                 } else {
                     const T d = diag_of(wx, wy, wz, nx, ny, nz, per, i, t.j, t.k, c);
-                    v = d > T(0) ? omega * relax_div(-b[c], d) : T(0);
+                    v = relaxable(d) ? omega * relax_div(-b[c], d) : T(0);
                 }
             } else {
                 const T xc = x[c];
                 T d, f;
                 stencil(wx, wy, wz, LoadPlain<T>{x}, nx, ny, nz, per, i, t.j, t.k, c, xc, d, f);
                 if (di) v = di[c] > T(0) ? xc + omega * ((f - b[c]) * di[c]) : xc;  // (rows of other than whole quads)
-                else v = d > T(0) ? xc + omega * relax_div(f - b[c], d) : xc;
+                else v = relaxable(d) ? xc + omega * relax_div(f - b[c], d) : xc;
             }
             x[c] = v;
             if constexpr (OUT) add_outer<T>(po, (int)c, v);

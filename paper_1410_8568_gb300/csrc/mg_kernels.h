@@ -111,20 +111,26 @@ template <class T> void launch_half_rows(const Table &, int colour, double omega
                                          const OuterView *ov, cudaStream_t);
 template <class T> void launch_restrict_rows(const Table &, double omega, cudaStream_t);
 template <class T> void launch_prolong_rows(const Table &, const OuterView *ov, cudaStream_t);
-// one-pass red-black sweep (mg_fused.cu, and mg_staged.cu for the staged
-// shapes): shape v fits a level with n cells per axis and periodic bits per in
-// FP32 (fp32) or FP64 cycles; sweep_layout fills the view's strip and chunk
-// fields for shape v and returns the blocks of the grid; a launch reads the
-// iterate from x (dir 0) or x2 (dir 1) and writes the other buffer; flags as
-// for the half-sweep (kHalfZero, kHalfOuter)
+// one-pass red-black sweep (mg_fused.cu: whole rows; mg_march.cu: variants 7 and
+// up): shape v fits a level with n cells per axis and periodic bits per in FP32
+// (fp32) or FP64 cycles; sweep_layout fills the view's strip and chunk fields for
+// shape v and returns the blocks of the grid; a launch reads the iterate from x
+// (dir 0) or x2 (dir 1) and writes the other buffer; flags as for the half-sweep
+// (kHalfZero, kHalfOuter)
+constexpr int kMarchVariant = 7;  // launch_sweep: this and above march
 bool sweep_fits(const int n[3], int per, int v, bool fp32);
-bool staged_fits(const int n[3], int per);
-int staged_layout(LevelView &v, int kc);
-void launch_sweep_staged(const Table &, int dir, double omega, int flags, const OuterView *ov, cudaStream_t);
 int sweep_layout(LevelView &v, int variant);
 int sweep_blocks(const int n[3], int variant);
 template <class T> void launch_sweep(const Table &, int dir, double omega, int flags, const OuterView *ov,
                                      cudaStream_t);
+// the marching one-pass sweep of FP32 cycles (mg_march.cu) on levels with rows of
+// whole quads: march_chunk gives the planes per block (0: half-sweeps are
+// faster); staged_fits: the levels the public shapes 7 .. 10 are offered for
+bool march_fits(const int n[3], int per);
+bool staged_fits(const int n[3], int per);
+int march_chunk(const int n[3], int per);
+int march_layout(LevelView &v, int kc);
+void launch_march(const Table &, int dir, double omega, int flags, const OuterView *ov, cudaStream_t);
 // V-cycle stages below the row-tiled levels; cyc as Table::cyc
 // (the tail: FP32 cycles, mg_tail.cu; tail_floats: shared-memory elements of its
 // level t of nt with N cells)

@@ -63,11 +63,28 @@ __device__ __forceinline__ void stq(T *p, const Quad<T> &q)
     }
 }
 
+// num / den for a den in the normal range.  FP32 (inner cycles): the 1-ulp
+// reciprocal and a product, within 2 ulp of the quotient, two instructions;
+// the approximate division of the same accuracy also scales subnormal and huge
+// divisors, in eight, which the issue-bound sweeps feel.
 template <class T>
 __device__ __forceinline__ T relax_div(T num, T den)
 {
-    if constexpr (sizeof(T) == 4) return __fdividef(num, den);  // inner cycle: 2-ulp division
-    else return num / den;
+    if constexpr (sizeof(T) == 4) {
+        float r;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(den));
+        return num * r;
+    } else {
+        return num / den;
+    }
+}
+// a diagonal that a cell can be relaxed with: positive (FP32: and normal; cells
+// of a smaller one would carry corrections beyond the FP32 range)
+template <class T>
+__device__ __forceinline__ bool relaxable(T d)
+{
+    if constexpr (sizeof(T) == 4) return d >= 1.17549435e-38f;
+    else return d > T(0);
 }
 
 // half-sweep flags: the iterate is zero on entry (first red launch); the
@@ -106,7 +123,7 @@ __device__ __forceinline__ T relax_cell(T xc, T xl, T xr, T fl, T fr, T fs, T fn
     f = fma(fn, xn - xc, f);
     f = fma(fb, xb - xc, f);
     f = fma(ft, xt - xc, f);
-    return d > T(0) ? fma(omega, relax_div(f - bc, d), xc) : xc;
+    return relaxable(d) ? fma(omega, relax_div(f - bc, d), xc) : xc;
 }
 
 // The relaxation of FP64 cycles, with the cell's diagonal given by its inverse
@@ -306,6 +323,14 @@ __device__ __forceinline__ T prolong_at(const T *__restrict__ ec, const int nc[3
     return lin(y0, y1);
 }
 
+// quotient of the coefficient-weighted means (any positive divisor)
+template <class T>
+__device__ __forceinline__ T mean_div(T num, T den)
+{
+    if constexpr (sizeof(T) == 4) return __fdividef(num, den);
+    else return num / den;
+}
+
 // Flux-conserving prolongation (Sec. 2.3 item 4, Eqs. 13-14) at one fine cell.
 // e[q], a[q]: coarse error and cell coefficient of the 8 coarse cells around
 // the fine centre, q = bit 0 (x partner) | bit 1 (y partner) | bit 2 (z partner),
@@ -328,9 +353,9 @@ __device__ __forceinline__ T flux_corner_mean(const T e[8], const T a[8])
     const T s0246 = s02 + (ae[4] + ae[6]), d0246 = d02 + (a[4] + a[6]);
     const T s_all = s0123 + ((ae[4] + ae[5]) + (ae[6] + ae[7]));
     const T d_all = d0123 + ((a[4] + a[5]) + (a[6] + a[7]));
-    const T fx = relax_div(s01, d01), fy = relax_div(s02, d02), fz = relax_div(s04, d04);
-    const T exy = relax_div(s0123, d0123), exz = relax_div(s0145, d0145), eyz = relax_div(s0246, d0246);
-    const T node = relax_div(s_all, d_all);
+    const T fx = mean_div(s01, d01), fy = mean_div(s02, d02), fz = mean_div(s04, d04);
+    const T exy = mean_div(s0123, d0123), exz = mean_div(s0145, d0145), eyz = mean_div(s0246, d0246);
+    const T node = mean_div(s_all, d_all);
     return T(0.125) * (((e[0] + fx) + (fy + fz)) + ((exy + exz) + (eyz + node)));
 }
 
@@ -424,7 +449,7 @@ __device__ __forceinline__ T zero_start_red(const LevelView &L, int I, int J, in
     d += wz[c];
     if (K + 1 < nz) d += wz[c + sz];
     else if (per & 4) d += wz[c - sz * (nz - 1)];
-    return d > T(0) ? omega * relax_div(-bc, d) : T(0);
+    return relaxable(d) ? omega * relax_div(-bc, d) : T(0);
 }
 
 template <class T>

@@ -122,7 +122,7 @@ __device__ __forceinline__ void item_setup(const TailView &V, int t, int q, cons
     // first cell: faces fx.x (low x), fx.y; second: fx.y, fe
     const float d0 = ((((f.fx.x + f.fx.y) + f.fs.x) + f.fn.x) + f.fb.x) + f.ft.x;
     const float d1 = ((((f.fx.y + f.fe) + f.fs.y) + f.fn.y) + f.fb.y) + f.ft.y;
-    const float i0 = d0 > 0.f ? relax_div(omega, d0) : 0.f, i1 = d1 > 0.f ? relax_div(omega, d1) : 0.f;
+    const float i0 = relaxable(d0) ? relax_div(omega, d0) : 0.f, i1 = relaxable(d1) ? relax_div(omega, d1) : 0.f;
     const bool p = s.p;
     o.fo = f.fx.y;
     o.rf = p ? f.fe : f.fx.x;

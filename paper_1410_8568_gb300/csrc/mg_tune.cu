@@ -257,17 +257,25 @@ int time_sweep(mg_handle *h, int v, float *ms)
     return MG_OK;
 }
 
-// Finest-level sweep: MG_SWEEP_HALF, a forced one-pass shape, or the fastest
-// of the half-sweep pair and every one-pass shape that fits (cached like the
-// launch shapes).
+// Sweeps: MG_SWEEP_HALF, a forced one-pass shape, a cached choice, the marching
+// sweep where its rule picks it, or the fastest of the half-sweep pair and every
+// whole-row shape that fits (cached like the launch shapes).
 int tune_sweep(mg_handle *h)
 {
     h->tile[MG_TILE_SWEEP][0] = 0;
+    memset(h->mkc, 0, sizeof(h->mkc));
+    // levels below the finest with a second buffer march (see onepass_possible)
+    for (int l = 1; l + 1 < h->L; l++)
+        if (h->lev[l].x2 && l < first_tail_level(h)) h->mkc[l] = march_chunk(h->lev[l].n, h->per);
     if (!h->lev[0].x2 || h->L < 2 || first_tail_level(h) < 1) return MG_OK;
     const int *n = h->lev[0].n;
     const int forced = h->prm.sweep;
+    auto choose = [h](int v) {
+        h->tile[MG_TILE_SWEEP][0] = (signed char)v;
+        h->mkc[0] = sweep_shape(v).tile_x ? sweep_shape(v).Kc : 0;
+    };
     if (forced >= 0) {
-        h->tile[MG_TILE_SWEEP][0] = (signed char)((forced > 0 && sweep_fits(n, h->per, forced, h->mixed)) ? forced : 0);
+        choose((forced > 0 && sweep_fits(n, h->per, forced, h->mixed)) ? forced : 0);
         return MG_OK;
     }
     TuneKey key;
@@ -281,15 +289,26 @@ int tune_sweep(mg_handle *h)
         env_cache_locked();
         auto it = g_tune.find(key);
         if (it != g_tune.end()) {
-            h->tile[MG_TILE_SWEEP][0] = (signed char)it->second;
+            choose(it->second);
             return MG_OK;
         }
+    }
+    // the marching sweep by rule, in chunks of its own (reported as the shape
+    // whose chunks hold them); where it is not the faster one, the half-sweep
+    // pair against the whole-row shapes, timed
+    const int kc = h->mixed ? march_chunk(n, h->per) : 0;
+    if (kc) {
+        h->mkc[0] = kc;
+        int v = kMarchVariant;
+        while (v + 1 < kSweepVariants && sweep_shape(v).Kc < kc) v++;
+        h->tile[MG_TILE_SWEEP][0] = (signed char)v;
+        return MG_OK;
     }
     float t[kSweepVariants];
     for (int v = 0; v < kSweepVariants; v++) t[v] = -1.f;
     for (int round = 0; round < 3; round++)
         for (int v = 0; v < kSweepVariants; v++) {
-            if (v > 0 && !sweep_fits(n, h->per, v, h->mixed)) continue;
+            if (v > 0 && (v >= kMarchVariant || !sweep_fits(n, h->per, v, h->mixed))) continue;
             float ms = 0.f;
             const int rc = h->mixed ? time_sweep<float>(h, v, &ms) : time_sweep<double>(h, v, &ms);
             if (rc) return rc;
