@@ -487,6 +487,7 @@ int Plan::fill(mg_handle *const *handles, int count)
         v.xq = make_fastdiv(v.n[0] >= 4 ? (unsigned)(v.n[0] >> 2) : 1u);
         v.xy = make_fastdiv((unsigned)v.n[1]);
         v.dxt = make_fastdiv((unsigned)fine_xtiles(v.n[0]));
+        outer_march(v);
         for (int q = 0; q < 3; q++) {
             v.xp3[q] = h->xp3[q];
             v.w32[q] = h->xp ? h->lev[0].w32[q] : nullptr;

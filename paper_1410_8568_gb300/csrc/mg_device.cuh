@@ -216,6 +216,11 @@ struct OuterView {
     int xp;
     FastDiv xq, xy;      // division by the quads per row n[0] / 4 and by n[1]
     FastDiv dxt;         // division by the row tiles of a row, fine_xtiles(n[0])
+    // march_pairs: items, planes per piece, log2 of a block's z pieces, tiles of
+    // pairs per plane; division by them and by the pairs of a row (0 items: rows of
+    // an odd number of cells)
+    int mitems, mkz, msub, mtiles;
+    FastDiv mdt, mdx;
     float *xp3[3];
     float *xb[2];
     const float *w32[3];
@@ -291,6 +296,35 @@ __host__ __device__ inline int outer_blocks(const int n[3])
 {
     const int t = fine_blocks(n);
     return t < kOuterCap ? t : kOuterCap;
+}
+// The pieces of a grid that its outer_blocks march (march_pairs): tiles of up to
+// 256 pairs of a plane and pieces of mkz planes, as long as they can be (a piece
+// reads one plane more and takes one difference more a cell) with the blocks
+// evenly loaded: the fewest planes on the busiest block, a piece counted as one
+// plane more; fewer, longer pieces unless shorter ones save 3 %.
+inline void outer_march(OuterView &v)
+{
+    v.mitems = 0;
+    v.mkz = v.mtiles = 1;
+    v.msub = 0;
+    if (v.n[0] % 2 == 0) {
+        const int pairs = (v.n[0] / 2) * v.n[1];
+        while (v.msub < 3 && pairs <= (kThreads >> (v.msub + 1))) v.msub++;
+        const int tile = kThreads >> v.msub;
+        v.mtiles = (pairs + tile - 1) / tile;
+        long long best = 0;
+        for (int kz = v.n[2]; kz >= 1; kz = kz > 64 ? kz / 2 : kz - 1) {
+            const int chunks = (v.n[2] + (kz << v.msub) - 1) / (kz << v.msub), items = v.mtiles * chunks;
+            const long long cost = (long long)((items + v.nblk - 1) / v.nblk) * (kz + 1);
+            if (best == 0 || cost * 100 < best * 97) {
+                best = cost;
+                v.mkz = kz;
+                v.mitems = items;
+            }
+        }
+    }
+    v.mdt = make_fastdiv((unsigned)v.mtiles);
+    v.mdx = make_fastdiv(v.n[0] >= 2 ? (unsigned)(v.n[0] / 2) : 1u);
 }
 // Blocks of a launch over the cells of a coarse level (32 coarse cells per warp row).
 __host__ __device__ inline int coarse_xtiles(int nx) { return (nx + kCSeg - 1) / kCSeg; }

@@ -834,54 +834,32 @@ __global__ void k_begin(const OuterView *__restrict__ ov)
 }
 
 // Partial sums of the caller's right-hand side (which = 0, partial slot 3) or
-// of the iterate p (which = 1, slot 1), FP64.
+// of the iterate p (which = 1, slot 1), FP64.  (The right-hand side may be
+// 8-byte aligned: read by single values.)
 __global__ void __launch_bounds__(kThreads) k_sum(const OuterView *__restrict__ ov,
                                                   const int *__restrict__ start, int count, int which)
 {
     dep_entry();
     const int e = find_entry(start, count);
-    const OuterView O = ov[e];
+    const OuterView &O = ov[e];
     const int lb = blockIdx.x - start[e];
-    const int ntiles = fine_blocks(O.n);
-    const double *src = which == 0 ? O.b : O.p;
-    // end of an extended-precision solve that took a step: the iterate is the
-    // three-float one (summed in its internal scale)
-    const bool conv = which == 1 && xp_live(O);
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    // kUnroll tiles of the block's grid-stride sequence per pass: every load of
-    // the pass is issued before the additions, which then run in the order of
-    // the sequence (one tile after the other, two cells per tile)
-    for (int tile = lb; tile < ntiles; tile += kUnroll * O.nblk) {
-        double val[kUnroll][2];
-#pragma unroll
-        for (int u = 0; u < kUnroll; u++) {
-            const int tu = tile + u * O.nblk;
-            const Tile t = fine_tile(O.n, tu < ntiles ? tu : tile, O.dxt, O.xy);
-            const long long rowoff = (long long)O.n[0] * t.row;
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int i = t.xbase + (threadIdx.x & 31) + 32 * h;
-                const bool in = tu < ntiles && t.ok && i < O.n[0];
-                const long long c = rowoff + i;
-                double x = 0.0;
-                if (in) x = conv ? ((double)O.xp3[0][c] + (double)O.xp3[1][c]) + (double)O.xp3[2][c] : src[c];
-                val[u][h] = in ? x : 0.0;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kUnroll; u++) {
-            const int tu = tile + u * O.nblk;
-            if (tu >= ntiles) break;
-            const Tile t = fine_tile(O.n, tu, O.dxt, O.xy);
-            if (!t.ok) continue;
-#pragma unroll
-            for (int h = 0; h < 2; h++)
-                if (t.xbase + (threadIdx.x & 31) + 32 * h < O.n[0]) v[0] += val[u][h];
-        }
+    double v[1] = {0.0};
+    auto add = [&](int, double2 x, bool) { v[0] += x.x + x.y; };
+    if (which == 0) {
+        for_pairs(
+            O, lb, [&](int c, bool both) { return make_double2(O.b[c], both ? O.b[c + 1] : 0.0); }, add);
+    } else if (xp_live(O)) {
+        // end of an extended-precision solve that took a step: the iterate is the
+        // three-float one (summed in its internal scale)
+        auto one = [&](int c) { return ((double)O.xp3[0][c] + (double)O.xp3[1][c]) + (double)O.xp3[2][c]; };
+        for_pairs(
+            O, lb, [&](int c, bool both) { return make_double2(one(c), both ? one(c + 1) : 0.0); }, add);
+    } else {
+        for_pairs(
+            O, lb, [&](int c, bool both) { return both ? ld2(O.p + c) : make_double2(O.p[c], 0.0); }, add);
     }
-    double out[4];
-    block_sum4(v, out);
-    if (threadIdx.x == 0) O.part[kPart * lb + (which == 0 ? 3 : 1)] = out[0];
+    block_sum(v);
+    if (threadIdx.x == 0) O.part[kPart * lb + (which == 0 ? 3 : 1)] = v[0];
 }
 
 // ---- extended-precision outer iteration (mixed-precision multigrid) --------
@@ -911,51 +889,37 @@ __global__ void __launch_bounds__(kThreads) k_center_rhs(const OuterView *__rest
 {
     dep_entry();
     const int e = find_entry(start, count);
-    const OuterView O = ov[e];
+    const OuterView &O = ov[e];
     if (!O.st->active) return;
     const int lb = blockIdx.x - start[e];
-    const int ntiles = fine_blocks(O.n);
     const double m = O.st->bmean;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    int nz = 0;
-    // loads of kUnroll tiles first, then the sequence's arithmetic in order (see k_sum)
-    for (int tile = lb; tile < ntiles; tile += kUnroll * O.nblk) {
-        double bv[kUnroll][2], pv[kUnroll][2];
-#pragma unroll
-        for (int u = 0; u < kUnroll; u++) {
-            const int tu = tile + u * O.nblk;
-            const Tile t = fine_tile(O.n, tu < ntiles ? tu : tile, O.dxt, O.xy);
-            const long long rowoff = (long long)O.n[0] * t.row;
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int i = t.xbase + (threadIdx.x & 31) + 32 * h;
-                const bool in = tu < ntiles && t.ok && i < O.n[0];
-                bv[u][h] = in ? O.b[rowoff + i] : 0.0;
-                pv[u][h] = in ? O.p[rowoff + i] : 0.0;
+    double v[1] = {0.0};
+    // a nonzero p by its bits (all but the sign; a NaN's are not zero either)
+    unsigned long long nz = 0;
+    struct In {
+        double2 b, p;
+    };
+    for_pairs(
+        O, lb,
+        [&](int c, bool both) {
+            if (both) return In{make_double2(O.b[c], O.b[c + 1]), ld2(O.p + c)};
+            return In{make_double2(O.b[c], 0.0), make_double2(O.p[c], 0.0)};
+        },
+        [&](int c, const In &x, bool both) {
+            const double b0 = x.b.x - m, b1 = x.b.y - m;
+            v[0] = fma(b0, b0, v[0]);
+            nz |= (unsigned long long)__double_as_longlong(x.p.x) << 1;
+            if (both) {
+                v[0] = fma(b1, b1, v[0]);
+                nz |= (unsigned long long)__double_as_longlong(x.p.y) << 1;
+                *reinterpret_cast<double2 *>(O.b0 + c) = make_double2(b0, b1);
+            } else {
+                O.b0[c] = b0;
             }
-        }
-#pragma unroll
-        for (int u = 0; u < kUnroll; u++) {
-            const int tu = tile + u * O.nblk;
-            if (tu >= ntiles) break;
-            const Tile t = fine_tile(O.n, tu, O.dxt, O.xy);
-            if (!t.ok) continue;
-            const long long rowoff = (long long)O.n[0] * t.row;
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int i = t.xbase + (threadIdx.x & 31) + 32 * h;
-                if (i >= O.n[0]) continue;
-                const double bc = bv[u][h] - m;
-                O.b0[rowoff + i] = bc;
-                v[2] += bc * bc;
-                nz |= !(pv[u][h] == 0.0);
-            }
-        }
-    }
-    double out[4];
-    block_sum4(v, out);
-    if (__syncthreads_or(nz) && threadIdx.x == 0) atomicOr(&O.st->pnz, 1);
-    if (threadIdx.x == 0) O.part[kPart * lb + 2] = out[2];
+        });
+    block_sum(v);
+    if (__syncthreads_or(nz != 0) && threadIdx.x == 0) atomicOr(&O.st->pnz, 1);
+    if (threadIdx.x == 0) O.part[kPart * lb + 2] = v[0];
 }
 
 // Scaled right-hand side and iterate in their float forms.
@@ -1141,73 +1105,132 @@ __global__ void __launch_bounds__(kThreads) k_residual_xp(const OuterView *__res
             }
         }
     }
-    double v[4] = {(double)racc, 0.0, 0.0, 0.0};
-    double out[4];
-    block_sum4(v, out);
-    if (threadIdx.x == 0) O.part[kPart * lb + 0] = out[0];
+    double v[1] = {(double)racc};
+    block_sum(v);
+    if (threadIdx.x == 0) O.part[kPart * lb + 0] = v[0];
 }
 #undef XP_FACE
 
+// r scaled by 2^k in the cycles' precision: the exponent moved and the
+// significand rounded (to nearest, ties to even) in integer arithmetic, as the
+// product and the F2F conversion are FP64-pipe operations; values that are not
+// normal before and after take those, in a function of its own (inlined, the
+// compiler predicates them and every cell issues them).
+__device__ __noinline__ double scaled_slow(double r, int k) { return r * __hiloint2double((1023 + k) << 20, 0); }
+__device__ __noinline__ float scaled_slow_f(double r, int k) { return (float)(r * __hiloint2double((1023 + k) << 20, 0)); }
+__device__ __forceinline__ void scaled(double r, int k, float &out)
+{
+    const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r), mag = hi & 0x7fffffffu;
+    const int ex = (int)(mag >> 20), es = ex + k - 896;  // float exponent field
+    if (ex == 0 || ex == 2047 || es < 1 || es > 253) {
+        // (a zero stays one)
+        out = (mag | lo) == 0u ? __uint_as_float(hi) : scaled_slow_f(r, k);
+        return;
+    }
+    unsigned b = ((unsigned)es << 23) | ((mag & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned rem = lo & 0x1fffffffu, half = 0x10000000u;
+    b += (rem > half || (rem == half && (b & 1u))) ? 1u : 0u;
+    out = __uint_as_float(b | (hi & 0x80000000u));
+}
+__device__ __forceinline__ void scaled(double r, int k, double &out)
+{
+    const int hi = __double2hiint(r), ex = (int)(((unsigned)hi & 0x7fffffffu) >> 20);
+    if (ex == 0 || ex == 2047 || ex + k < 1 || ex + k > 2046) out = scaled_slow(r, k);
+    else out = __hiloint2double(hi + (k << 20), __double2loint(r));
+}
+
 // Outer residual r = (b - mean b) - A p in FP64, handed to the V-cycle in its
-// precision Te, scaled by xscale (a power of 2; 1 for CG).  init = 1 (start of
-// a CG solve): also stores b0 = b - mean(b) and the partial sums of ||b0||^2
-// (slot 2), all FP64.  init = 2 (start of a multigrid iteration): as 0, but a
-// grid whose starting iterate is zero everywhere (GridState::pnz clear) takes
-// r = b0 without evaluating A p, which is exactly zero there.  ||r||^2 goes to
-// slot 0; after the first CG residual it is accumulated from the rounded,
-// scaled r handed to the cycle (a norm only steers the stopping test, so its
-// own rounding at 1e-7 relative is immaterial, and the scale keeps FP32
-// squares inside the FP32 range).
-template <class Te>
-__global__ void __launch_bounds__(kThreads) k_residual(const OuterView *__restrict__ ov,
-                                                       const int *__restrict__ start, int count,
-                                                       int init)
+// precision Te, scaled by xscale (a power of 2; 1 for CG).  INIT (start of a CG
+// solve): also stores b0 = b - mean(b) and the partial sums of ||b0||^2 (slot 2),
+// all FP64.  first (start of a multigrid iteration): a grid whose starting
+// iterate is zero everywhere (GridState::pnz clear) takes r = b0 without
+// evaluating A p, which is exactly zero there.  ||r||^2 goes to slot 0; after the
+// first CG residual it is accumulated from the rounded, scaled r handed to the
+// cycle (a norm only steers the stopping test, so its own rounding at 1e-7
+// relative is immaterial, and the scale keeps FP32 squares inside the FP32 range).
+//
+// Bound by the FP64 pipe: 10.5 operations a cell (march_pairs) against 15 with
+// each cell's six differences, b - f, the scale and the conversion for itself.
+template <class Te, bool INIT>
+__global__ void __launch_bounds__(kThreads, 4) k_residual(const OuterView *__restrict__ ov,
+                                                          const int *__restrict__ start, int count, int first)
 {
     dep_entry();
     const int e = find_entry(start, count);
-    const OuterView O = ov[e];
+    const OuterView &O = ov[e];
     const GridState *s = O.st;
     if (!s->active) return;
     const int lb = blockIdx.x - start[e];
-    const int ntiles = fine_blocks(O.n);
-    const int nx = O.n[0];
     Te *r = (Te *)O.r;
-    const double m = s->bmean, sc = s->xscale;
-    const bool cold = init == 2 && !s->pnz;
-    if (init == 2) init = 0;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    const double m = s->bmean;
+    const int ksc = ((__double2hiint(s->xscale) >> 20) & 2047) - 1023;
+    const bool cold = first && !s->pnz;
+    double v[INIT ? 2 : 1] = {};
     Te racc = Te(0);
-    for (int tile = lb; tile < ntiles; tile += O.nblk) {
-        const Tile t = fine_tile(O.n, tile, O.dxt, O.xy);
-        if (!t.ok) continue;
-        const long long rowoff = (long long)nx * t.row;
-        for (int h = 0; h < 2; h++) {
-            const int i = t.xbase + (threadIdx.x & 31) + 32 * h;
-            if (i >= nx) continue;
-            const long long c = rowoff + i;
-            const double f = cold ? 0.0 : flux64(O, O.p, i, t.j, t.k, c);
+    if (cold) {
+        for_pairs(
+            O, lb, [&](int c, bool both) { return both ? ld2(O.b0 + c) : make_double2(O.b0[c], 0.0); },
+            [&](int c, double2 b, bool both) {
+                Te r0, r1;
+                scaled(b.x, ksc, r0);
+                scaled(b.y, ksc, r1);
+                r[c] = r0;
+                racc += r0 * r0;
+                if (both) {
+                    r[c + 1] = r1;
+                    racc += r1 * r1;
+                }
+            });
+    } else if (O.mitems) {
+        march_pairs(
+            O, O.p, lb,
+            [&](int c) {
+                if constexpr (!INIT) return ld2(O.b0 + c);
+                const double b0 = O.b[c] - m, b1 = O.b[c + 1] - m;
+                *reinterpret_cast<double2 *>(O.b0 + c) = make_double2(b0, b1);
+                v[INIT ? 1 : 0] = fma(b0, b0, v[INIT ? 1 : 0]);
+                v[INIT ? 1 : 0] = fma(b1, b1, v[INIT ? 1 : 0]);
+                return make_double2(b0, b1);
+            },
+            [&](int c, double s0, double s1, double2) {
+                Te r0, r1;
+                scaled(s0, ksc, r0);
+                scaled(s1, ksc, r1);
+                r[c] = r0;
+                r[c + 1] = r1;
+                if (O.r64) *reinterpret_cast<double2 *>(O.r64 + c) = make_double2(s0, s1);  // CG keeps the FP64 residual
+                if constexpr (INIT) {
+                    v[0] = fma(s0, s0, v[0]);
+                    v[0] = fma(s1, s1, v[0]);
+                } else {
+                    racc += r0 * r0;
+                    racc += r1 * r1;
+                }
+            });
+    } else {
+        for_cells(O, lb, [&](int c, int i, int j, int k) {
             double bc;
-            if (init) {
+            if constexpr (INIT) {
                 bc = O.b[c] - m;
                 O.b0[c] = bc;
-                v[2] += bc * bc;
+                v[INIT ? 1 : 0] += bc * bc;
             } else {
                 bc = O.b0[c];
             }
-            const double rc = bc - f;
-            const Te rt = (Te)(rc * sc);
+            const double rc = bc - flux64(O, O.p, i, j, k, c);
+            Te rt;
+            scaled(rc, ksc, rt);
             r[c] = rt;
-            if (O.r64) O.r64[c] = rc;  // conjugate gradients keep the FP64 residual
-            if (init) v[0] += rc * rc;
+            if (O.r64) O.r64[c] = rc;
+            if constexpr (INIT) v[0] += rc * rc;
             else racc += rt * rt;
-        }
+        });
     }
-    if (!init) v[0] = (double)racc;
-    double out[4];
-    block_sum4(v, out);
+    if (!INIT) v[0] = (double)racc;
+    block_sum(v);
     if (threadIdx.x == 0) {
-        O.part[kPart * lb + 0] = out[0];
-        if (init) O.part[kPart * lb + 2] = out[2];
+        O.part[kPart * lb + 0] = v[0];
+        if (INIT) O.part[kPart * lb + 2] = v[INIT ? 1 : 0];
     }
 }
 
@@ -1223,25 +1246,35 @@ __global__ void __launch_bounds__(kThreads) k_finalize(const OuterView *__restri
     const OuterView &O = ov[blockIdx.x];
     GridState *s = O.st;
     if (mode != 3 && !s->active) return;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int q = threadIdx.x; q < O.nblk; q += blockDim.x)
-        for (int f = 0; f < 4; f++) v[f] += O.part[kPart * q + f];
-    double out[4];
-    block_sum4(v, out);
+    // the mode's sum (CG's starting residual kernel also reduced b)
+    const int slot = mode == 0 ? 3 : mode == 3 ? 1 : mode == 4 ? 2 : 0;
+    const bool two = mode == 1 && O.r64;
+    double v[2] = {0.0, 0.0};
+    for (int q = threadIdx.x; q < O.nblk; q += blockDim.x) {
+        v[0] += O.part[kPart * q + slot];
+        if (two) v[1] += O.part[kPart * q + 2];
+    }
+    if (two) {
+        block_sum(v);
+    } else {
+        double v0[1] = {v[0]};
+        block_sum(v0);
+        v[0] = v0[0];
+    }
     if (threadIdx.x != 0) return;
     const double N = (double)O.n[0] * O.n[1] * O.n[2];
     if (mode == 0) {
-        s->bmean = out[3] / N;
+        s->bmean = v[0] / N;
         return;
     }
     if (mode == 3) {
-        s->xmean = out[1] / N;
+        s->xmean = v[0] / N;
         return;
     }
     if (mode == 4) {
         // extended precision: ||b - mean b|| and the internal scale 2^-k,
         // 2^k near the rms of b - mean b (k kept inside the FP32 exponent range)
-        s->bnorm = sqrt(out[2]);
+        s->bnorm = sqrt(v[0]);
         const double rms = s->bnorm / sqrt(N);
         int k = (rms > 0.0 && isfinite(rms)) ? ilogb(rms) : 0;
         k = k < -100 ? -100 : (k > 100 ? 100 : k);
@@ -1250,10 +1283,10 @@ __global__ void __launch_bounds__(kThreads) k_finalize(const OuterView *__restri
         return;
     }
     // the partials are of the scaled residual (xscale = 1 for CG)
-    const double rn = sqrt(out[0]) * s->xinv;
+    const double rn = sqrt(v[0]) * s->xinv;
     int done = 0;
     if (mode == 1) {
-        if (O.r64) s->bnorm = sqrt(out[2]);  // CG: the starting residual kernel also reduced b
+        if (O.r64) s->bnorm = sqrt(v[1]);
         s->r0 = rn;
     } else {
         done = s->cycles_next;
@@ -1294,29 +1327,26 @@ __global__ void __launch_bounds__(kThreads) k_final(const OuterView *__restrict_
 {
     dep_entry();
     const int e = find_entry(start, count);
-    const OuterView O = ov[e];
+    const OuterView &O = ov[e];
     const GridState *s = O.st;
     const int lb = blockIdx.x - start[e];
-    const int ntiles = fine_blocks(O.n);
     const double m = s->xmean;
     const bool zero = s->bnorm == 0.0;
     const bool conv = xp_live(O);
     const double inv = conv ? 1.0 / s->xscale : 1.0;  // a power of 2: exact
-    for (int tile = lb; tile < ntiles; tile += O.nblk) {
-        const Tile t = fine_tile(O.n, tile, O.dxt, O.xy);
-        if (!t.ok) continue;
-        const long long rowoff = (long long)O.n[0] * t.row;
-        for (int h = 0; h < 2; h++) {
-            const int i = t.xbase + (threadIdx.x & 31) + 32 * h;
-            if (i >= O.n[0]) continue;
-            const long long c = rowoff + i;
-            double v;
-            if (zero) v = 0.0;
-            else if (conv) v = ((((double)O.xp3[0][c] - m) + (double)O.xp3[1][c]) + (double)O.xp3[2][c]) * inv;
-            else v = O.p[c] - m;
-            O.p[c] = v;
-        }
-    }
+    auto one = [&](int c) { return ((((double)O.xp3[0][c] - m) + (double)O.xp3[1][c]) + (double)O.xp3[2][c]) * inv; };
+    for_pairs(
+        O, lb,
+        [&](int c, bool both) {
+            if (conv) return make_double2(one(c), both ? one(c + 1) : 0.0);
+            return both ? ld2(O.p + c) : make_double2(O.p[c], 0.0);
+        },
+        [&](int c, double2 p, bool both) {
+            if (!conv) p = make_double2(p.x - m, p.y - m);
+            if (zero) p = make_double2(0.0, 0.0);
+            if (both) *reinterpret_cast<double2 *>(O.p + c) = p;
+            else O.p[c] = p.x;
+        });
 }
 
 // Loop control of a graph-driven solve: keep iterating while any grid of the
@@ -1472,7 +1502,8 @@ void launch_sum(const OuterTable &ot, int which, cudaStream_t s)
 template <class Te>
 void launch_residual(const OuterTable &ot, int init, cudaStream_t s)
 {
-    launch_k(k_residual<Te>, ot.blocks, kThreads, 0, s, ot.ov, ot.start, ot.count, init);
+    if (init == 1) launch_k(k_residual<Te, true>, ot.blocks, kThreads, 0, s, ot.ov, ot.start, ot.count, 0);
+    else launch_k(k_residual<Te, false>, ot.blocks, kThreads, 0, s, ot.ov, ot.start, ot.count, init == 2 ? 1 : 0);
 }
 void launch_center_rhs(const OuterTable &ot, cudaStream_t s)
 {
