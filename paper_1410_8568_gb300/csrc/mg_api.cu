@@ -105,7 +105,7 @@ struct Layout {
     size_t x2[MG_MAX_LEVELS];  // second iterate buffer (one-pass sweep), 0 if none
     size_t dinv[MG_MAX_LEVELS];  // FP64 cycles: inverse diagonals of the relaxed levels (0 if none)
     size_t alpha64[MG_MAX_LEVELS], alpha32[MG_MAX_LEVELS];
-    size_t G, b0, part, err, state, dstate, dview, dstart, dcview, setup_cv, total;
+    size_t G, b0, part, err, state, dstate, dview, dstart, dcview, total;
     size_t pcg[4];
     size_t xp3[3], xb[2], wlo[3];  // extended-precision outer iteration
     bool xp;
@@ -171,7 +171,6 @@ static int plan_layout(const mg_grid &g, const mg_params &p, Layout &lay)
     lay.dview = c.take(sizeof(LevelView));
     lay.dstart = c.take(2 * sizeof(int));
     lay.dcview = c.take(sizeof(CoarseView));
-    lay.setup_cv = c.take(sizeof(CoarseView));
     lay.total = c.off;
     return MG_OK;
 }
@@ -402,7 +401,7 @@ int Plan::fill(mg_handle *const *handles, int count)
     ot = OuterTable{ov, d_starts + so0, G, starts[nst - 1]};
     tail_smem = 0;
     ntv = 0;
-    ncv = 0;
+    ncv = cv_most = 0;
     cv_dense = cv_gmres = false;
     for (int g = 0; g < G; g++) {
         mg_handle *h = hs[g];
@@ -459,6 +458,7 @@ int Plan::fill(mg_handle *const *handles, int count)
         v.gm_tol = h->prm.coarse_tol;
         if (h->gmres) cv_gmres = true;
         else cv_dense = true;
+        if (!h->gmres) cv_most = std::max(cv_most, v.nc);
     }
     for (int g = 0; g < G; g++) {
         mg_handle *h = hs[g];
@@ -609,7 +609,7 @@ static void vcycle(Plan &P, Prof &pf, int cyc, bool outer)
     }
     if (P.ncv) {
         pf.begin(s, MG_K_COARSE, P.Lmax - 1);
-        if (P.cv_dense) launch_coarse_solve<T>(P.cv, P.ncv, cyc, outer ? P.ov : nullptr, s);
+        if (P.cv_dense) launch_coarse_solve<T>(P.cv, P.ncv, P.cv_most, cyc, outer ? P.ov : nullptr, s);
         if (P.cv_gmres) launch_coarse_gmres<T>(P.cv, P.ncv, cyc, outer ? P.ov : nullptr, s);
         pf.end(s);
     }
@@ -1059,7 +1059,7 @@ static int upload_faces(mg_handle *h)
         a.dy = make_fastdiv((unsigned)a.n[1]);
         launch_diag_inv(a, h->stream);
     }
-    if (!h->gmres) launch_coarse_setup(h->setup_cv, 1, h->stream);
+    if (!h->gmres) launch_coarse_setup(h->setup_view, h->stream);
     CK(cudaGetLastError());
     return MG_OK;
 }
@@ -1178,7 +1178,6 @@ int gbmg::handle_alloc(const mg_grid *grid, const mg_params *params, void *strea
     h->dview = (LevelView *)(h->slab + lay.dview);
     h->dstart = (int *)(h->slab + lay.dstart);
     h->dcview = (CoarseView *)(h->slab + lay.dcview);
-    h->setup_cv = (CoarseView *)(h->slab + lay.setup_cv);
     GridState ds;
     memset(&ds, 0, sizeof(ds));
     ds.active = 1;
@@ -1189,8 +1188,7 @@ int gbmg::handle_alloc(const mg_grid *grid, const mg_params *params, void *strea
     {
         // view of the coarsest level for building its inverse (mg_create / mg_set_faces)
         const HLevel &Cl = h->lev[h->L - 1];
-        CoarseView v;
-        memset(&v, 0, sizeof(v));
+        CoarseView &v = h->setup_view;
         for (int d = 0; d < 3; d++) {
             v.n[d] = Cl.n[d];
             v.w[d] = Cl.w64[d];
@@ -1199,7 +1197,6 @@ int gbmg::handle_alloc(const mg_grid *grid, const mg_params *params, void *strea
         v.nc = (int)Cl.N;
         v.G = h->G;
         v.err = h->err + 1;
-        CK(cudaMemcpy(h->setup_cv, &v, sizeof(v), cudaMemcpyHostToDevice));
     }
     rc = tune_handle(h);
     if (rc) {
@@ -1764,8 +1761,8 @@ int mg_coarse_solve(mg_handle *h, int prec, const void *r, void *e)
         if (prec == MG_PREC_MIXED) launch_coarse_gmres<float>(h->dcview, 1, 0, nullptr, h->stream);
         else launch_coarse_gmres<double>(h->dcview, 1, 0, nullptr, h->stream);
     } else {
-        if (prec == MG_PREC_MIXED) launch_coarse_solve<float>(h->dcview, 1, 0, nullptr, h->stream);
-        else launch_coarse_solve<double>(h->dcview, 1, 0, nullptr, h->stream);
+        if (prec == MG_PREC_MIXED) launch_coarse_solve<float>(h->dcview, 1, v.nc, 0, nullptr, h->stream);
+        else launch_coarse_solve<double>(h->dcview, 1, v.nc, 0, nullptr, h->stream);
     }
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(h->stream));

@@ -82,7 +82,7 @@ struct mg_handle {
     gbmg::LevelView *dview = nullptr;    // view slot of the unit calls
     int *dstart = nullptr;
     gbmg::CoarseView *dcview = nullptr;
-    gbmg::CoarseView *setup_cv = nullptr;  // coarsest level, for building its inverse
+    gbmg::CoarseView setup_view = {};  // coarsest level, for building its inverse
     char *slab = nullptr;
     size_t bytes = 0;
     gbmg::Plan *plan = nullptr;          // single-grid launch plan
@@ -127,6 +127,7 @@ struct Plan {
     Table sweep[MG_MAX_LEVELS]; // one-pass sweeps of level l (count 0: half-sweeps)
     CoarseView *cv = nullptr;   // coarsest solves of the grids without a tail
     int ncv = 0;
+    int cv_most = 0;  // cells of the largest dense coarsest grid
     bool cv_dense = false, cv_gmres = false;  // which coarse kernels the cv table needs
     TailView *tv = nullptr;     // bottom-of-cycle blocks of the grids with a tail
     int ntv = 0;

@@ -29,7 +29,7 @@
 // order, so the result is deterministic.
 #include "mg_kernels.h"
 #include "mg_stencil.cuh"
-#include "mg_bulk.cuh"  // smem_u32
+#include "mg_cluster.cuh"
 
 #include <math.h>
 
@@ -45,33 +45,6 @@ constexpr int kGmSmem = kGmCells * (10 * 8 + 6 * 4);            // r, p, q, d, 6
 constexpr int kGmRestarts = 8;
 static_assert(kGmPer * kGmThreads == kGmCells, "whole threads");
 static_assert(kGmSmem + 3 * kGmThreads * 8 + 1024 <= 232448, "shared memory of one block");
-
-__device__ __forceinline__ unsigned cluster_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ unsigned map_rank(unsigned addr, unsigned rank)
-{
-    unsigned a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ double ld_cluster(unsigned addr)
-{
-    double v;
-    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_cluster(unsigned addr, double v)
-{
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
-}
 
 struct GmScratch {
     double part[3][kGmThreads];       // one value per thread

@@ -433,131 +433,6 @@ __global__ void __launch_bounds__(kThreads) k_apply(const LevelView *__restrict_
 }
 
 // ---------------------------------------------------------------------------
-// (6) coarsest grid: exact solve e = -G b with G = (-A + c 1 1^T)^{-1}
-// ---------------------------------------------------------------------------
-
-// For sum(b) = 0 this is the zero-mean solution of A e = b; for sum(b) != 0 it
-// solves A e = b - mean(b) and adds a constant, which the cycle ignores
-// (A 1 = 0) and the final mean removal takes out.  One warp per row of G
-// (rows are contiguous, G is symmetric), lanes split the dot product, fixed
-// shuffle tree.  A grid whose finest level is its coarsest (C.outer) adds e
-// to its FP64 iterate in the last cycle of a refinement step (ov non-null).
-template <class T>
-__global__ void __launch_bounds__(kThreads) k_coarse_solve(const CoarseView *__restrict__ cv, int cyc,
-                                                           const OuterView *__restrict__ ov)
-{
-    dep_entry();
-    const CoarseView &C = cv[blockIdx.x];
-    if (C.gmres || !in_cycle(C.st, cyc)) return;  // GMRES grids: k_coarse_gmres
-    __shared__ double rb[kMaxCoarse];
-    const int n = C.nc;
-    const T *b = (const T *)C.b;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) rb[t] = (double)b[t];
-    __syncthreads();
-    T *x = (T *)C.x;
-    const bool out = ov != nullptr && C.outer && last_cycle(C.st, cyc);
-    const OuterOut po = out ? outer_out(ov[C.g]) : OuterOut{};
-    const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-    for (int t = threadIdx.x >> 5; t < n; t += warps) {
-        const double *Gt = C.G + (long long)t * n;
-        double s = 0.0;
-        for (int u = lane; u < n; u += 32) s += Gt[u] * rb[u];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-            const T xn = (T)(-s);
-            x[t] = xn;
-            if (out) add_outer<T>(po, t, xn);
-        }
-    }
-}
-
-// Assemble S = -A + c 1 1^T of the coarsest level (c = mean diagonal / n, so the
-// constant vector becomes an eigenvector with a mid-spectrum eigenvalue) and
-// invert it in place by Gauss-Jordan elimination.  S is symmetric positive
-// definite, so no pivoting is needed; a non-positive pivot means the grid is
-// cut into pieces by zero coefficients and raises *err.
-__global__ void __launch_bounds__(1024) k_coarse_setup(const CoarseView *__restrict__ cv)
-{
-    dep_entry();
-    const CoarseView &C = cv[blockIdx.x];
-    const int n = C.nc;
-    const int nx = C.n[0], ny = C.n[1], nz = C.n[2];
-    double *S = C.G;
-    __shared__ double col[kMaxCoarse];
-    __shared__ double red[32];
-    __shared__ double c0;
-    __shared__ int bad;
-    for (long long q = threadIdx.x; q < (long long)n * n; q += blockDim.x) S[q] = 0.0;
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
-    double dsum = 0.0;
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        const int i = c % nx, j = (c / nx) % ny, k = c / (nx * ny);
-        const int q[3] = {i, j, k};
-        const int nn[3] = {nx, ny, nz};
-        const long long stride[3] = {1, nx, (long long)nx * ny};
-        double diag = 0.0;
-        for (int d = 0; d < 3; d++) {
-            // low face
-            if (q[d] > 0 || (C.per >> d & 1)) {
-                const double a = C.w[d][c];
-                const long long nb = q[d] > 0 ? c - stride[d] : c + stride[d] * (nn[d] - 1);
-                if (nb != c) {
-                    diag += a;
-                    S[(long long)c * n + nb] -= a;
-                }
-            }
-            // high face
-            if (q[d] + 1 < nn[d] || (C.per >> d & 1)) {
-                const long long fc = q[d] + 1 < nn[d] ? c + stride[d] : c - stride[d] * (nn[d] - 1);
-                const double a = C.w[d][fc];
-                if (fc != c) {
-                    diag += a;
-                    S[(long long)c * n + fc] -= a;
-                }
-            }
-        }
-        S[(long long)c * n + c] += diag;
-        dsum += diag;
-    }
-    // deterministic block sum of the diagonal
-    for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = dsum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += red[w];
-        c0 = s / n / n;
-    }
-    __syncthreads();
-    for (long long q = threadIdx.x; q < (long long)n * n; q += blockDim.x) S[q] += c0;
-    __syncthreads();
-    const int warps = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int k = 0; k < n; k++) {
-        for (int r = threadIdx.x; r < n; r += blockDim.x) col[r] = S[(long long)r * n + k];
-        __syncthreads();
-        const double piv = col[k];
-        if (!(piv > 0.0)) {
-            if (threadIdx.x == 0) bad = 1;
-            __syncthreads();
-            break;
-        }
-        for (int j = threadIdx.x; j < n; j += blockDim.x)
-            S[(long long)k * n + j] = (j == k ? 1.0 : S[(long long)k * n + j]) / piv;
-        __syncthreads();
-        for (int r = wid; r < n; r += warps) {
-            if (r == k) continue;
-            const double f = col[r];
-            double *Sr = S + (long long)r * n;
-            const double *Sk = S + (long long)k * n;
-            for (int j = lane; j < n; j += 32) Sr[j] = (j == k ? 0.0 : Sr[j]) - f * Sk[j];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && bad) *C.err = 1;
-}
-
-// ---------------------------------------------------------------------------
 // coefficients: density -> faces (2), caller faces -> scaled level-0 faces,
 // and coarse faces
 // ---------------------------------------------------------------------------
@@ -1448,15 +1323,6 @@ void launch_apply(const Table &tb, cudaStream_t s)
 {
     launch_k(k_apply<T>, tb.blocks, kThreads, 0, s, tb.lv, tb.start, tb.count);
 }
-template <class T>
-void launch_coarse_solve(const CoarseView *cv, int count, int cyc, const OuterView *ov, cudaStream_t s)
-{
-    launch_k(k_coarse_solve<T>, count, kThreads, 0, s, cv, cyc, ov);
-}
-void launch_coarse_setup(const CoarseView *cv, int count, cudaStream_t s)
-{
-    launch_k(k_coarse_setup, count, 1024, 0, s, cv);
-}
 static int cells_grid(long long N)
 {
     long long b = (N + kThreads - 1) / kThreads;
@@ -1534,8 +1400,6 @@ template void launch_prolong_rows<float>(const Table &, const OuterView *, cudaS
 template void launch_prolong_rows<double>(const Table &, const OuterView *, cudaStream_t);
 template void launch_apply<float>(const Table &, cudaStream_t);
 template void launch_apply<double>(const Table &, cudaStream_t);
-template void launch_coarse_solve<float>(const CoarseView *, int, int, const OuterView *, cudaStream_t);
-template void launch_coarse_solve<double>(const CoarseView *, int, int, const OuterView *, cudaStream_t);
 template void launch_residual<float>(const OuterTable &, int, cudaStream_t);
 template void launch_residual<double>(const OuterTable &, int, cudaStream_t);
 

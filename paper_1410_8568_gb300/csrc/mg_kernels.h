@@ -137,11 +137,11 @@ void launch_march(const Table &, int dir, double omega, int flags, const OuterVi
 int tail_floats(int N, int t, int nt, bool flux);
 void launch_tail(const TailView *, int count, size_t smem, double omega, int nu1, int nu2, int cyc, cudaStream_t);
 template <class T> void launch_apply(const Table &, cudaStream_t);
-template <class T> void launch_coarse_solve(const CoarseView *, int count, int cyc, const OuterView *ov,
+template <class T> void launch_coarse_solve(const CoarseView *, int count, int most, int cyc, const OuterView *ov,
                                             cudaStream_t);
 template <class T> void launch_coarse_gmres(const CoarseView *, int count, int cyc, const OuterView *ov,
                                             cudaStream_t);
-void launch_coarse_setup(const CoarseView *, int count, cudaStream_t);
+void launch_coarse_setup(const CoarseView &, cudaStream_t);
 void launch_faces_from_density(const FaceArgs &, cudaStream_t);
 void launch_scale_faces(const FaceArgs &, cudaStream_t);
 void launch_coarsen_faces(const CoarsenArgs &, cudaStream_t);
