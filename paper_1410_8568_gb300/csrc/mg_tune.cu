@@ -45,10 +45,17 @@ namespace gbmg {
 // below the finest with at most kTailCells cells, if at least one level above
 // the coarsest qualifies (else the grid has no tail: L).  FP32 cycles only: one
 // block per grid runs at one SM's FP64 rate, which on this GPU is far below
-// that of the per-level FP64 kernels spread over all SMs.
+// that of the per-level FP64 kernels spread over all SMs.  For the same reason
+// a coarsest grid above kTailCoarse cells is solved by its own launch (n^2 FP64
+// multiply-adds, a block per 8 rows; 385 cells: 39 us in one block), although the
+// launches of the levels above it come back with it.  A solve with and without
+// the tail, us: 175 coarsest cells (56 x 40 x 40) 730, 748; 225 (40 x 40 x 72) 947,
+// 898; 343 (56^3) 1051, 785; 385 (56 x 40 x 88) 1818, 1217.
+constexpr long long kTailCoarse = 200;
 int first_tail_level(const mg_handle *h)
 {
     if (!h->mixed || h->gmres) return h->L;  // the tail solves the coarsest grid with its inverse
+    if ((long long)h->lev[h->L - 1].N > kTailCoarse) return h->L;
     for (int l = 1; l + 1 < h->L && l < MG_MAX_LEVELS; l++)
         if (h->lev[l].N <= kTailCells && h->L - l <= kMaxTail) return l;
     return h->L;

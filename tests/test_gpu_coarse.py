@@ -47,3 +47,33 @@ def test_coarse_solve_residual(shape, bc):
         S.set_density(rho)
         S.coarse_solve(b, again, prec=gbmg.FP64)
         assert torch.equal(e, again)
+
+
+@pytest.mark.parametrize("shape", [
+    (56, 40, 40),   # 175 coarsest cells: the bottom of the cycle in one block
+    (40, 40, 72),   # 225: a launch per level and the solve by its own launch
+    (56, 56, 36),   # 14 x 14 x 9: GMRES
+    (40, 56, 88),   # 385
+])
+def test_solve_alone_and_in_a_batch(shape):
+    """Converged (the solver's own FP64 residual) and the same bits next to a grid
+    that keeps the one-block bottom."""
+    rng = np.random.default_rng(shape[0] + shape[2])
+    probs = []
+    for sh in (shape, (32, 32, 32)):
+        rho = torch.from_numpy(np.exp(rng.uniform(0.0, np.log(10.0), size=sh[::-1]))).cuda()
+        b = torch.from_numpy(rng.standard_normal(sh[::-1])).cuda()
+        probs.append((sh, rho, b - b.mean()))
+    alone = []
+    for sh, rho, b in probs:
+        with gbmg.Solver(sh, (0, 0, 0), rho=rho, max_iters=100) as S:
+            p = torch.zeros_like(b)
+            st = S.solve(b, p, tol=1e-10)
+            assert st.rel_res <= 1e-10
+            alone.append(p)
+    solvers = [gbmg.Solver(sh, (0, 0, 0), rho=rho, max_iters=100) for sh, rho, _ in probs]
+    ps = [torch.zeros_like(b) for _, _, b in probs]
+    B = gbmg.Batch(solvers)
+    B.solve([b for _, _, b in probs], ps, tol=1e-10)
+    for p, q in zip(ps, alone):
+        assert torch.equal(p, q)
