@@ -241,6 +241,9 @@ def count_launches(shape, iters, steps, nu1=2, nu2=2, inner=3, tail_cells=4096, 
         per_step = 3 + (1 if inner > 1 else 0)  # residual, finalize, loop control (+ step control)
     epilogue = 3                       # sum p, mean, p - mean
     # (below the finest level the first red half-sweep was not a launch of its own)
+    # (one launch per sweep; on the finest level the outer iterate's update is a launch of its own)
+    if 0 in onepass and not pcg:
+        per_step += 1
     for l in onepass if not pcg else ():
         if l < normal:
             cycle -= nu1 + nu2 - (1 if l > 0 else 0)

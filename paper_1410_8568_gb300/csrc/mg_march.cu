@@ -135,9 +135,8 @@ __device__ __forceinline__ void copy16(unsigned dst, const float *src)
 // test for walls.  Lanes and rows beyond the tile repeat the work of a lane of
 // the same parity (same values to the same places); only the stores of own
 // cells are guarded.
-template <bool ZERO, bool OUT>
-__device__ __forceinline__ void march_body(const LevelView &L, int lb, int dir, float omega, const OuterOut &po,
-                                           March &sh)
+template <bool ZERO>
+__device__ __forceinline__ void march_body(const LevelView &L, int lb, int dir, float omega, March &sh)
 {
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
     const float *__restrict__ xin = (const float *)(dir ? L.x2 : L.x);
@@ -290,7 +289,6 @@ __device__ __forceinline__ void march_body(const LevelView &L, int lb, int dir, 
             o.v[1 - PAR] = B.r.x;
             o.v[3 - PAR] = B.r.y;
             stq(xout + c, o);
-            if constexpr (OUT) add_outer_quad<float>(po, c, o.v, 0xF);
         }
         sh.red[cur][me] = red;
         // plane k becomes plane k - 1
@@ -345,51 +343,102 @@ __device__ __forceinline__ void march_body(const LevelView &L, int lb, int dir, 
     }
 }
 
-template <bool MAYOUT>
-__device__ __forceinline__ void march_entry(const LevelView &L, int lb, int dir, float omega, int flags, int cyc,
-                                            const OuterView *__restrict__ ov)
+__device__ __forceinline__ void march_entry(const LevelView &L, int lb, int dir, float omega, int flags, int cyc)
 {
     extern __shared__ __align__(16) unsigned char march_smem[];
     March &sh = *(March *)march_smem;
     // the whole block returns together (a grid's state is uniform)
     if (!in_cycle(L.st, cyc)) return;
-    if constexpr (MAYOUT) {  // the last post-sweep of a cycle, never the first of one
-        if (last_cycle(L.st, cyc)) {
-            march_body<false, true>(L, lb, dir, omega, outer_out(ov[L.g]), sh);
-            return;
-        }
-    } else if (flags & kZeroGuess) {
-        march_body<true, false>(L, lb, dir, omega, OuterOut{}, sh);
-        return;
-    }
-    march_body<false, false>(L, lb, dir, omega, OuterOut{}, sh);
+    if (flags & kZeroGuess) march_body<true>(L, lb, dir, omega, sh);
+    else march_body<false>(L, lb, dir, omega, sh);
 }
 
-template <bool MAYOUT>
-__global__ void __launch_bounds__(32 * W, 1) k_march(const LevelView *__restrict__ lv,
-                                                                      const int *__restrict__ start, int count,
-                                                                      int dir, float omega, int flags, int cyc,
-                                                                      const OuterView *__restrict__ ov,
-                                                                      const __grid_constant__ LevelView one,
-                                                                      int single)
+__global__ void __launch_bounds__(32 * W, 1) k_march(const LevelView *__restrict__ lv, const int *__restrict__ start,
+                                                     int count, int dir, float omega, int flags, int cyc,
+                                                     const __grid_constant__ LevelView one, int single)
 {
     dep_entry();
     if (single) {
-        march_entry<MAYOUT>(one, blockIdx.x, dir, omega, flags, cyc, ov);
+        march_entry(one, blockIdx.x, dir, omega, flags, cyc);
         return;
     }
     const int e = find_entry(start, count);
-    march_entry<MAYOUT>(lv[e], blockIdx.x - start[e], dir, omega, flags, cyc, ov);
+    march_entry(lv[e], blockIdx.x - start[e], dir, omega, flags, cyc);
 }
 
-template <bool MAYOUT>
-void launch_march_b(const Table &tb, int dir, double omega, int flags, const OuterView *ov, cudaStream_t s)
+// p + v 2^sh (|sh| <= 500), with the conversion and the scaling on the bits of v:
+// they and a multiply-add would be two FP64 operations a cell, the addition is one.
+__device__ __forceinline__ double add_shifted(double p, float v, int sh)
 {
-    static const cudaError_t opt_in = cudaFuncSetAttribute(
-        k_march<MAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(March));
-    (void)opt_in;
-    launch_k(k_march<MAYOUT>, tb.blocks, 32 * W, sizeof(March), s, tb.lv, tb.start, tb.count, dir, (float)omega, flags,
-             tb.cyc, ov, table_view(tb), table_single(tb));
+    const bool small = (__float_as_uint(v) & 0x7fffffffu) < 0x00800000u;  // zero or subnormal
+    const unsigned b = __float_as_uint(small ? __fmul_rn(v, 0x1p64f) : v), m = b & 0x7fffffffu;
+    unsigned e = (m >> 3) + ((unsigned)(896 + sh - (small ? 64 : 0)) << 20);
+    if (m >= 0x7f800000u) e = (m >> 3) + (1792u << 20);  // infinite, not a number
+    if (m == 0u) e = 0u;
+    return p + __hiloint2double((int)((b & 0x80000000u) | e), (int)(b << 29));
+}
+
+// The correction of the grids whose step ends with this cycle into their outer
+// iterates, by the blocks of the sweep before it (block lb of nb of a grid takes
+// every nb-th piece).  Bound by HBM: 20 B a cell, 432 us at 512^3 (6.2 TB/s).  With
+// the update in the sweep's own stores, which left no register to ask for the
+// iterate ahead of time, that sweep took 1175 us instead of 507; staging the iterate
+// in shared memory as well left no L1 for what spilled, 1198 us.
+__device__ __forceinline__ void outer_entry(const LevelView &L, int lb, int nb, int dir, int cyc,
+                                            const OuterView *__restrict__ ov)
+{
+    if (!in_cycle(L.st, cyc) || !last_cycle(L.st, cyc)) return;
+    const OuterOut po = outer_out(ov[L.g]);
+    const float *__restrict__ x = (const float *)(dir ? L.x : L.x2);
+    const int quads = L.n[0] * L.n[1] * L.n[2] >> 2, step = nb * 32 * W;
+    const int hi = __double2hiint(po.inv), sh = (hi >> 20) - 1023;
+    // an FP64 iterate and a scale of 2^sh
+    const bool shifted = po.t[0] == nullptr && (hi & 0xfffff) == 0 && __double2loint(po.inv) == 0 && sh >= -500 && sh <= 500;
+    int q = lb * 32 * W + (int)threadIdx.x;
+    if (!shifted) {
+        for (; q < quads; q += step) {
+            const float4 v = ldg4(x + 4 * q);
+            const float e[4] = {v.x, v.y, v.z, v.w};
+            add_outer_quad<float>(po, 4 * q, e, 0xF);
+        }
+        return;
+    }
+    double2 *__restrict__ p = (double2 *)po.p;
+    constexpr int U = 4;  // quads of a thread in flight
+    for (; q < quads; q += U * step) {
+        float4 v[U];
+        double2 a[U], d[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int c = q + u * step;
+            if (c < quads) {
+                v[u] = ldg4(x + 4 * c);
+                a[u] = p[2 * c];
+                d[u] = p[2 * c + 1];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int c = q + u * step;
+            if (c < quads) {
+                p[2 * c] = make_double2(add_shifted(a[u].x, v[u].x, sh), add_shifted(a[u].y, v[u].y, sh));
+                p[2 * c + 1] = make_double2(add_shifted(d[u].x, v[u].z, sh), add_shifted(d[u].y, v[u].w, sh));
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(32 * W) k_outer_add(const LevelView *__restrict__ lv, const int *__restrict__ start,
+                                                      int count, int dir, int cyc, const OuterView *__restrict__ ov,
+                                                      const __grid_constant__ LevelView one, int single)
+{
+    dep_entry();
+    if (single) {
+        outer_entry(one, blockIdx.x, gridDim.x, dir, cyc, ov);
+        return;
+    }
+    const int e = find_entry(start, count);
+    outer_entry(lv[e], blockIdx.x - start[e], start[e + 1] - start[e], dir, cyc, ov);
 }
 
 
@@ -463,8 +512,14 @@ int march_layout(LevelView &v, int kc)
 void launch_march(const Table &tb, int dir, double omega, int flags, const OuterView *ov, cudaStream_t s)
 {
     if (tb.blocks == 0) return;
-    if (flags & kOuter) launch_march_b<true>(tb, dir, omega, flags, ov, s);
-    else launch_march_b<false>(tb, dir, omega, flags, nullptr, s);
+    static const cudaError_t opt_in =
+        cudaFuncSetAttribute(k_march, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(March));
+    (void)opt_in;
+    launch_k(k_march, tb.blocks, 32 * W, sizeof(March), s, tb.lv, tb.start, tb.count, dir, (float)omega, flags, tb.cyc,
+             table_view(tb), table_single(tb));
+    if (flags & kOuter)
+        launch_k(k_outer_add, tb.blocks, 32 * W, 0, s, tb.lv, tb.start, tb.count, dir, tb.cyc, ov, table_view(tb),
+                 table_single(tb));
 }
 
 }  // namespace gbmg

@@ -67,3 +67,19 @@ def test_batch_shares_the_launch():
     B.close()
     for S in solvers:
         S.close()
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-30, 1e30])
+def test_outer_iterate_at_any_scale(scale):
+    """The last sweep of a step adds the correction times a power of 2 to the
+    caller's iterate, on the bits of the correction: the same bits as by
+    multiply-adds."""
+    P = I.config2(128)
+    rhs = torch.from_numpy(P.rhs).cuda() * scale
+    got = []
+    for sweep in (gbmg.SWEEP_HALF, gbmg.SWEEP_AUTO):
+        p = torch.zeros_like(rhs)
+        with gbmg.Solver(P.shape, P.bc, rho=torch.from_numpy(P.rho).cuda(), sweep=sweep) as S:
+            assert S.solve(rhs, p, tol=1e-10).status == gbmg.OK
+        got.append(p)
+    assert torch.equal(*got)
