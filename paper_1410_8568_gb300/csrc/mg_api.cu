@@ -329,6 +329,18 @@ int Plan::fill(mg_handle *const *handles, int count)
                 if (!tile_fits(h->lev[l].n, var[k])) var[k] = 0;
         }
         if (flux) var[MG_TILE_PROLONG] = 0;
+        // FP64 restrictions of few cells (any variant gives the same bits)
+        if (!mixed && prm.tiles == MG_TILES_AUTO) {
+            bool quads = true;
+            long long coarse = 0;
+            for (int g = 0; g < G; g++) {
+                mg_handle *h = hs[g];
+                if (l + 1 >= h->L || l >= lt[g]) continue;
+                quads = quads && (h->lev[l].n[0] & 3) == 0;
+                coarse += (long long)h->lev[l + 1].N;
+            }
+            if (quads && coarse <= kSplitCells) var[MG_TILE_RESTRICT] = kSplitVariant;
+        }
         // without post-smoothing the finest level's prolongation also updates the
         // outer iterate, in the row-tiled kernel (launch_prolong): its blocks
         if (l == 0 && prm.nu2 == 0) var[MG_TILE_PROLONG] = 0;

@@ -95,6 +95,10 @@ int restrict_blocks(const int n[3], const int nc[3]);
 int prolong_blocks(const int n[3]);
 // the same for launch shape v (mg_tiles.cu); v > 0 needs n[0] % 4 == 0
 bool tile_fits(const int n[3], int v);
+// FP64 restriction tables of at most kSplitCells coarse cells: a lane per fine
+// row (k_restrict_split), Table::variant kSplitVariant
+constexpr int kSplitVariant = 64, kSplitThreads = 128;
+constexpr long long kSplitCells = 300000;
 int half_sweep_blocks_v(const int n[3], int v);
 int restrict_blocks_v(const int n[3], const int nc[3], int v);
 int prolong_blocks_v(const int n[3], const int nc[3], int v);

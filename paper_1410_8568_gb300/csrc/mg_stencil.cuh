@@ -408,12 +408,13 @@ __device__ __forceinline__ Quad<T> residual_quad(const T *__restrict__ x, const 
 #pragma unroll
     for (int u = 0; u < 4; u++) {
         const T xc = xq.v[u];
-        T f = fx.v[u] * ((u > 0 ? xq.v[u - 1] : xw) - xc);
-        f += (u < 3 ? fx.v[u + 1] : fxe) * ((u < 3 ? xq.v[u + 1] : xe) - xc);
-        f += fy.v[u] * (xs.v[u] - xc);
-        f += fyn.v[u] * (xn.v[u] - xc);
-        f += fz.v[u] * (xb.v[u] - xc);
-        f += fzt.v[u] * (xt.v[u] - xc);
+        // (every restriction kernel the same roundings)
+        T f = mul_rn(fx.v[u], (u > 0 ? xq.v[u - 1] : xw) - xc);
+        f = fma(u < 3 ? fx.v[u + 1] : fxe, (u < 3 ? xq.v[u + 1] : xe) - xc, f);
+        f = fma(fy.v[u], xs.v[u] - xc, f);
+        f = fma(fyn.v[u], xn.v[u] - xc, f);
+        f = fma(fz.v[u], xb.v[u] - xc, f);
+        f = fma(fzt.v[u], xt.v[u] - xc, f);
         r.v[u] = bq.v[u] - f;
     }
     return r;

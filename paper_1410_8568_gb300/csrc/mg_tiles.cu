@@ -107,6 +107,56 @@ __global__ void __launch_bounds__(B, 1024 / B) k_restrict_flat(const LevelView *
     restrict_flat_entry<T, B, Q>(lv[e], blockIdx.x - start[e], cyc, omega, false);
 }
 
+// FP64 restriction of few cells: restrict_pair with a lane per fine row's quad
+// instead of a thread for all four.  What bounds it is the chain of a thread's FP64
+// operations (12 a cell of the 4 x 4, 75 cycles each), not the memory or the pipe:
+// 17 us on levels of 64^3 down to 4^3 cells.  The two cells' sums run in the order
+// of restrict_pair, in the group's first two lanes.  An FP64 solve with it up to
+// 0, 40 000, 300 000 and 3 million coarse cells, us: 64^3 2870, 2320, 2290, 2280;
+// 128^3 7560, 7030, 6930, 6910; 192^3 18550, 18050, 17990, 18250.  In FP32, whose
+// chains are short: no difference up to 40 000, 128^3 1870 -> 1940 beyond; not used.
+__device__ __forceinline__ void restrict_split_entry(const LevelView &L, int lb, int cyc, double omega, bool defer)
+{
+    using T = double;
+    const bool go = in_cycle(L.st, cyc);
+    if (!defer && !go) return;
+    const int np = L.nc[0] >> 1, ncy = L.nc[1], items = np * ncy * L.nc[2];
+    const int t = lb * kSplitThreads + (int)threadIdx.x, q = t & 3, h = q & 1;
+    const int g = min(t >> 2, items - 1);  // (lanes beyond the last item repeat it: whole warps shuffle)
+    const int crow = fdiv(g, L.dp);
+    const int K = fdiv(crow, L.dcy), J = crow - K * ncy, P = g - crow * np;
+    const Quad<T> r = residual_quad((const T *)L.x, (const T *)L.b, (const T *)L.w[0], (const T *)L.w[1],
+                                    (const T *)L.w[2], L.n[0], L.n[1], L.n[2], L.per, 4 * P, 2 * J + h,
+                                    2 * K + (q >> 1));
+    T s = T(0);
+#pragma unroll
+    for (int m = 0; m < 4; m++) {
+        const T a = __shfl_sync(0xffffffffu, r.v[0], m, 4), b = __shfl_sync(0xffffffffu, r.v[1], m, 4),
+                c = __shfl_sync(0xffffffffu, r.v[2], m, 4), d = __shfl_sync(0xffffffffu, r.v[3], m, 4);
+        s += h ? c : a;
+        s += h ? d : b;
+    }
+    if (!go || q > 1 || (t >> 2) >= items) return;
+    const int c = L.nc[0] * crow + 2 * P + h;
+    const T bc = s * T(0.125);
+    ((T *)L.bc)[c] = bc;
+    if (L.zr) ((T *)L.xc)[c] = zero_start_red<T>(L, 2 * P + h, J, K, bc, omega);
+}
+
+__global__ void __launch_bounds__(kSplitThreads) k_restrict_split(const LevelView *__restrict__ lv,
+                                                                  const int *__restrict__ start, int count, int cyc,
+                                                                  double omega, const __grid_constant__ LevelView one,
+                                                                  int single)
+{
+    dep_entry();
+    if (single) {
+        restrict_split_entry(one, blockIdx.x, cyc, omega, true);
+        return;
+    }
+    const int e = find_entry(start, count);
+    restrict_split_entry(lv[e], blockIdx.x - start[e], cyc, omega, false);
+}
+
 // defer: see half_entry
 template <class T, int B, int Q>
 __device__ __forceinline__ void prolong_flat_entry(const LevelView &L, int lb, int cyc, bool defer)
@@ -184,6 +234,7 @@ int prolong_blocks_v(const int n[3], const int nc[3], int v)
 int restrict_blocks_v(const int n[3], const int nc[3], int v)
 {
     if (v == 0) return restrict_blocks(n, nc);
+    if (v == kSplitVariant) return (int)((2ll * nc[0] * nc[1] * nc[2] + kSplitThreads - 1) / kSplitThreads);
     return flat_blocks((long long)(nc[0] >> 1) * nc[1] * nc[2], v);
 }
 
@@ -207,6 +258,11 @@ template <class T>
 void launch_restrict(const Table &tb, double omega, cudaStream_t s)
 {
     if (tb.blocks == 0) return;
+    if (tb.variant == kSplitVariant) {  // (FP64 plans)
+        launch_k(k_restrict_split, tb.blocks, kSplitThreads, 0, s, tb.lv, tb.start, tb.count, tb.cyc, omega,
+                 table_view(tb), table_single(tb));
+        return;
+    }
     const bool flat = with_variant(tb.variant, [&](auto V) {
         constexpr TileShape ts = tile_shape(decltype(V)::value);
         launch_k(k_restrict_flat<T, ts.B, ts.Q>, tb.blocks, ts.B, 0, s, tb.lv, tb.start, tb.count, tb.cyc,
