@@ -363,8 +363,8 @@ __device__ __forceinline__ void prolong_body(const LevelView &L, int lb, const O
         const int i = t.xbase + (threadIdx.x & 31) + 32 * h;
         if (i >= nx) continue;
         const long long c = (long long)nx * t.row + i;
-        const T xn = x[c] + (FLUX ? prolong_at_flux(ec, (const T *)L.ac, L.nc, L.per, i, t.j, t.k)
-                                  : prolong_at(ec, L.nc, L.per, i, t.j, t.k));
+        const T xn = FLUX ? x[c] + prolong_at_flux(ec, (const T *)L.ac, L.nc, L.per, i, t.j, t.k)
+                          : add_lin(x[c], prolong_at(ec, L.nc, L.per, i, t.j, t.k));
         x[c] = xn;
         if constexpr (OUT) add_outer<T>(po, (int)c, xn);
     }

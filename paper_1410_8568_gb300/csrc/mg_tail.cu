@@ -264,6 +264,7 @@ __device__ __forceinline__ float coarse_rhs(const TailView &V, int t, const floa
 }
 
 // (4) the prolonged correction of level t + 1 at the two cells of the item at s
+// (trilinear: 64 times it, see lin)
 __device__ __forceinline__ float2 prolong_item(const TailView &V, int t, const Arr &C, const Pos &s)
 {
     const int ncx = V.n[t + 1][0], ncy = V.n[t + 1][1], per = V.per;
@@ -317,10 +318,12 @@ __device__ __forceinline__ void prolong_children(const TailView &V, int t, const
     e[3] = make_float2(lin(y1[1].x, y1[2].x), lin(y1[1].y, y1[2].y));
 }
 
-__device__ __forceinline__ void item_add(Item &it, int p, float2 e)
+// Adds the correction e of the pair's cells; flux: as it is, else 64 times it (lin).
+__device__ __forceinline__ void item_add(Item &it, int p, float2 e, bool flux)
 {
-    it.xr += p ? e.y : e.x;
-    it.xb += p ? e.x : e.y;
+    const float f = flux ? 1.f : 0.015625f;
+    it.xr = fmaf(f, p ? e.y : e.x, it.xr);
+    it.xb = fmaf(f, p ? e.x : e.y, it.xb);
 }
 __device__ __forceinline__ float2 item_cells(const Item &it, int p)
 {
@@ -513,7 +516,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailView *__rest
 #pragma unroll
             for (int u = 0; u < kItemWords; u++) w[u] = A.items[u * NI + tid];
             s = unpack_pos(A.pos[tid]);
-            item_add(it[0], s.p, prolong_item(V, t, level_arr(V, t + 1, sm), s));
+            item_add(it[0], s.p, prolong_item(V, t, level_arr(V, t + 1, sm), s), V.flux);
             A.R[tid] = it[0].xr;
             A.B[tid] = it[0].xb;
         }
@@ -540,7 +543,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailView *__rest
         }
 #pragma unroll
         for (int i = 0; i < kTailItems; i++) {
-            item_add(it0[i], (i ^ (i >> 1)) & 1, e[i]);
+            item_add(it0[i], (i ^ (i >> 1)) & 1, e[i], V.flux);
             A0.R[pl0[i]] = it0[i].xr;
             A0.B[pl0[i]] = it0[i].xb;
         }
