@@ -130,23 +130,26 @@ __device__ __forceinline__ T relax_cell(T xc, T xl, T xr, T fl, T fr, T fs, T fn
 // di = 1 / d (d summed as relax_cell sums it; 0 for a cell without faces),
 // computed once per coefficient set: the Gauss-Seidel value
 // g = (sum of w_f x_nb - b) di, then x = g (omega = 1) or xc + omega (g - xc).
-// Eight FP64 operations per cell at omega = 1 (six fused multiply-adds, a
-// subtraction, a multiply) where the difference form with a division takes
-// about thirty; this GPU issues FP64 on a narrow pipe, which bounds the FP64
-// half-sweep.  The neighbours are summed in relax_cell's order.
+// Seven FP64 operations per cell at omega = 1 (six fused multiply-adds, a
+// multiply) where the difference form with a division takes about thirty; this
+// GPU issues FP64 on a narrow pipe, which bounds the FP64 half-sweep.  The tests
+// are on the bits and the case omega != 1 is a call: as FP64 comparisons and
+// predicated operations they took the pipe too (a half-sweep of 128^3 26.4 us,
+// now 21.2 us).  The neighbours are summed in relax_cell's order.
+__device__ __noinline__ inline double over_relax(double xc, double g, double omega) { return fma(omega, g - xc, xc); }
 template <class T>
 __device__ __forceinline__ T relax_cell_inv(T xc, T xl, T xr, T fl, T fr, T fs, T fn, T fb, T ft, T xs,
                                             T xn, T xb, T xt, T bc, T omega, T di)
 {
-    T s = fl * xl;
+    T s = fma(fl, xl, -bc);
     s = fma(fr, xr, s);
     s = fma(fs, xs, s);
     s = fma(fn, xn, s);
     s = fma(fb, xb, s);
     s = fma(ft, xt, s);
-    const T g = (s - bc) * di;
-    if (!(di > T(0))) return xc;
-    return omega == T(1) ? g : fma(omega, g - xc, xc);
+    T g = s * di;
+    if (__double_as_longlong((double)omega) != 0x3ff0000000000000ll) g = (T)over_relax(xc, g, omega);
+    return __double_as_longlong((double)di) > 0 ? g : xc;
 }
 
 // Add the final correction v of cell c of a refinement step to the outer
@@ -411,13 +414,15 @@ __device__ __forceinline__ Quad<T> residual_quad(const T *__restrict__ x, const 
     const Quad<T> xb = has_b ? ldq(x + cb) : Z, xt = has_t ? ldq(x + ct) : Z;
     const T xw = has_w ? x[cw] : T(0), xe = has_e ? x[ce] : T(0);
     const T fxe = has_e ? wx[ce] : T(0);
+    // (x differences once each: a cell's west one is its neighbour's east one, negated)
+    const T d[5] = {xq.v[0] - xw, xq.v[1] - xq.v[0], xq.v[2] - xq.v[1], xq.v[3] - xq.v[2], xe - xq.v[3]};
     Quad<T> r;
 #pragma unroll
     for (int u = 0; u < 4; u++) {
         const T xc = xq.v[u];
         // (every restriction kernel the same roundings)
-        T f = mul_rn(fx.v[u], (u > 0 ? xq.v[u - 1] : xw) - xc);
-        f = fma(u < 3 ? fx.v[u + 1] : fxe, (u < 3 ? xq.v[u + 1] : xe) - xc, f);
+        T f = mul_rn(fx.v[u], -d[u]);
+        f = fma(u < 3 ? fx.v[u + 1] : fxe, d[u + 1], f);
         f = fma(fy.v[u], xs.v[u] - xc, f);
         f = fma(fyn.v[u], xn.v[u] - xc, f);
         f = fma(fz.v[u], xb.v[u] - xc, f);
