@@ -390,8 +390,8 @@ int mg_coarse_solve(mg_handle *h, int prec, const void *r, void *e);
  * layout above, > 0 off the walls) and right-hand side r (DEVICE), all in
  * FP64.  So e has zero mean exactly when sum(r) = 0.  It assembles
  * -A + c 1 1^T with c = trace(-A) / n^2, inverts it by Gauss-Jordan
- * elimination and applies the inverse, the arithmetic of the coarsest-grid
- * solve of a handle.
+ * elimination and applies the inverse: the solve of a handle's coarsest grid
+ * (whose inverse is built by sweeps of one triangle: equal up to rounding).
  *
  * Scratch: a 2 MiB array in the library's static device memory, held by every
  * device that loads the library until the process exits.  The first call on a

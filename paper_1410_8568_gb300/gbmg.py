@@ -199,7 +199,7 @@ def make_params(precision=MIXED, nu1=2, nu2=2, omega=1.0, max_iters=100, use_gra
 def sweep_shape(variant):
     """(threads per block, planes per block, tile_x) of one-pass sweep shape
     `variant`; tile_x = 0 for the whole-row shapes, else the cells along x of a
-    staged shape's tile (FP32 cycles only)."""
+    marching shape's tile (FP32 cycles only)."""
     a, b, c = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
     check(lib().mg_sweep_shape(int(variant), ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)),
           "mg_sweep_shape")
