@@ -451,7 +451,8 @@ int mg_projection_step(mg_handle *h, double *ux, double *uy, double *uz, double 
 #define MG_K_COARSE 3
 #define MG_K_RESIDUAL 4 /* the FP64 residual + norms (the update p += e is folded into the cycle) */
 #define MG_K_OTHER 5
-#define MG_K_TAIL 6 /* the levels of at most 4096 cells and the coarsest solve, one block per grid */
+#define MG_K_TAIL 6 /* the levels of at most 4096 cells and the coarsest solve (grids of up to 200
+                       coarsest cells), one block per grid */
 #define MG_K_RESIDUAL0 7 /* the starting residual of a solve (a zero starting iterate skips A p) */
 #define MG_K_KINDS 8
 
