@@ -1,5 +1,10 @@
 // mg_cluster.cuh -- blocks of a thread-block cluster: ranks, the barrier and
 // access to each other's shared memory.
+//
+// Another block's shared memory may be touched only between two cluster barriers:
+// the first access (ld_cluster, st_cluster) comes after a barrier that every block
+// has arrived at since it started, and a block leaves after a barrier that every
+// block arrives at behind its last access.
 #pragma once
 
 #include "mg_bulk.cuh"  // smem_u32

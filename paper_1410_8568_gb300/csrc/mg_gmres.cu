@@ -110,6 +110,7 @@ __global__ void __launch_bounds__(kGmThreads, 1) k_coarse_gmres(const CoarseView
     dep_entry();
     const CoarseView &C = cv[blockIdx.x / (unsigned)size];
     if (!C.gmres || !in_cycle(C.st, cyc)) return;  // uniform over the cluster
+    cluster_arrive();  // this block has started (waited for before the first remote access)
     extern __shared__ __align__(16) unsigned char gm_smem[];
     __shared__ GmScratch S;
     unsigned turn = 0;
@@ -139,6 +140,7 @@ __global__ void __launch_bounds__(kGmThreads, 1) k_coarse_gmres(const CoarseView
         }
         v[0] += (double)bt[c0 + u];
     }
+    cluster_wait();  // every block has started: its shared memory may be written
     cluster_sum(v, 1, S, turn, rank, (unsigned)size);  // (its cluster barrier publishes r)
     const double mean = v[0] / n;
     for (int u = tid; u < cells; u += kGmThreads) {
