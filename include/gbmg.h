@@ -297,7 +297,8 @@ int mg_server_create(size_t hbm_budget_bytes, int max_slots, const mg_params *pa
                      void *stream, mg_server **out);
 
 /* Queue a solve.  grid, the face coefficients ax/ay/az, rhs and p are as in
- * mg_create/mg_solve (DEVICE); they must stay valid and unmodified until
+ * mg_create/mg_solve (DEVICE; a p that is not 16-byte aligned is taken too, and
+ * solved by narrower loads); they must stay valid and unmodified until
  * mg_poll reports the ticket finished.  Returns MG_EBUDGET if the request can
  * never fit in the budget. */
 int mg_submit(mg_server *s, const mg_grid *grid, const double *ax, const double *ay,

@@ -996,7 +996,7 @@ int run_plan(Plan &P, Prof &pf, const double *const *rhs, double *const *p, cons
 {
     for (int g = 0; g < P.G; g++) {
         if (!rhs[g] || !p[g] || !(tol[g] >= 0.0)) return MG_EINVAL;
-        if (((uintptr_t)p[g] & 15) != 0) return MG_EINVAL;  // p is staged in 16-byte pieces
+        if (((uintptr_t)p[g] & 15) != 0) return MG_EINVAL;  // (the documented alignment)
         P.ov_h[g].b = rhs[g];
         P.ov_h[g].p = p[g];
         P.ov_h[g].tol = tol[g];

@@ -769,8 +769,9 @@ __global__ void __launch_bounds__(kThreads) k_sum(const OuterView *__restrict__ 
         for_pairs(
             O, lb, [&](int c, bool both) { return make_double2(one(c), both ? one(c + 1) : 0.0); }, add);
     } else {
+        const bool pairs = p_pairs(O);
         for_pairs(
-            O, lb, [&](int c, bool both) { return both ? ld2(O.p + c) : make_double2(O.p[c], 0.0); }, add);
+            O, lb, [&](int c, bool both) { return both ? ld_p(O, c, pairs) : make_double2(O.p[c], 0.0); }, add);
     }
     block_sum(v);
     if (threadIdx.x == 0) O.part[kPart * lb + (which == 0 ? 3 : 1)] = v[0];
@@ -808,6 +809,7 @@ __global__ void __launch_bounds__(kThreads) k_center_rhs(const OuterView *__rest
     const int lb = blockIdx.x - start[e];
     const double m = O.st->bmean;
     double v[1] = {0.0};
+    const bool pairs = p_pairs(O);
     // a nonzero p by its bits (all but the sign; a NaN's are not zero either)
     unsigned long long nz = 0;
     struct In {
@@ -816,7 +818,7 @@ __global__ void __launch_bounds__(kThreads) k_center_rhs(const OuterView *__rest
     for_pairs(
         O, lb,
         [&](int c, bool both) {
-            if (both) return In{make_double2(O.b[c], O.b[c + 1]), ld2(O.p + c)};
+            if (both) return In{make_double2(O.b[c], O.b[c + 1]), ld_p(O, c, pairs)};
             return In{make_double2(O.b[c], 0.0), make_double2(O.p[c], 0.0)};
         },
         [&](int c, const In &x, bool both) {
@@ -1095,7 +1097,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_residual(const OuterView *__res
                     racc += r1 * r1;
                 }
             });
-    } else if (O.mitems) {
+    } else if (O.mitems && p_pairs(O)) {
         march_pairs(
             O, O.p, lb,
             [&](int c) {
@@ -1246,19 +1248,19 @@ __global__ void __launch_bounds__(kThreads) k_final(const OuterView *__restrict_
     const int lb = blockIdx.x - start[e];
     const double m = s->xmean;
     const bool zero = s->bnorm == 0.0;
-    const bool conv = xp_live(O);
+    const bool conv = xp_live(O), pairs = p_pairs(O);
     const double inv = conv ? 1.0 / s->xscale : 1.0;  // a power of 2: exact
     auto one = [&](int c) { return ((((double)O.xp3[0][c] - m) + (double)O.xp3[1][c]) + (double)O.xp3[2][c]) * inv; };
     for_pairs(
         O, lb,
         [&](int c, bool both) {
             if (conv) return make_double2(one(c), both ? one(c + 1) : 0.0);
-            return both ? ld2(O.p + c) : make_double2(O.p[c], 0.0);
+            return both ? ld_p(O, c, pairs) : make_double2(O.p[c], 0.0);
         },
         [&](int c, double2 p, bool both) {
             if (!conv) p = make_double2(p.x - m, p.y - m);
             if (zero) p = make_double2(0.0, 0.0);
-            if (both) *reinterpret_cast<double2 *>(O.p + c) = p;
+            if (both) st_p(O, c, pairs, p);
             else O.p[c] = p.x;
         });
 }

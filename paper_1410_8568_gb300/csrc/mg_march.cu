@@ -392,8 +392,9 @@ __device__ __forceinline__ void outer_entry(const LevelView &L, int lb, int nb, 
     const float *__restrict__ x = (const float *)(dir ? L.x : L.x2);
     const int quads = L.n[0] * L.n[1] * L.n[2] >> 2, step = nb * 32 * W;
     const int hi = __double2hiint(po.inv), sh = (hi >> 20) - 1023;
-    // an FP64 iterate and a scale of 2^sh
-    const bool shifted = po.t[0] == nullptr && (hi & 0xfffff) == 0 && __double2loint(po.inv) == 0 && sh >= -500 && sh <= 500;
+    // an FP64 iterate of aligned pairs and a scale of 2^sh
+    const bool shifted = po.t[0] == nullptr && ((size_t)po.p & 15) == 0 && (hi & 0xfffff) == 0 &&
+                         __double2loint(po.inv) == 0 && sh >= -500 && sh <= 500;
     int q = lb * 32 * W + (int)threadIdx.x;
     if (!shifted) {
         for (; q < quads; q += step) {

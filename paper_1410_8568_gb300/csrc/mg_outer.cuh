@@ -42,6 +42,24 @@ __device__ __forceinline__ void block_sum(double (&v)[N])
 
 __device__ __forceinline__ double2 ld2(const double *p) { return *reinterpret_cast<const double2 *>(p); }
 
+// The caller's arrays lie at any double (mg_solve asks for a 16-byte p, a served
+// request need not have one): pairs of its iterate move as vectors only where
+// they are aligned (the same for every pair of a grid).
+__device__ __forceinline__ bool p_pairs(const OuterView &O) { return ((size_t)O.p & 15) == 0; }
+__device__ __forceinline__ double2 ld_p(const OuterView &O, int c, bool pairs)
+{
+    return pairs ? ld2(O.p + c) : make_double2(O.p[c], O.p[c + 1]);
+}
+__device__ __forceinline__ void st_p(const OuterView &O, int c, bool pairs, double2 v)
+{
+    if (pairs) {
+        *reinterpret_cast<double2 *>(O.p + c) = v;
+    } else {
+        O.p[c] = v.x;
+        O.p[c + 1] = v.y;
+    }
+}
+
 // Every cell of a grid once, two at a time: f(c, v, both) for cells c and, if
 // both, c + 1 (c even), v = load(c, both).  The pairs are dealt to the threads of
 // the grid's blocks in turn; a thread has the loads of kPairs of them in flight.
@@ -150,7 +168,7 @@ __device__ __forceinline__ Tile fine_tile(const int n[3], int lb, const FastDiv 
 }
 
 // Sum over the 6 faces of w_f (x_nb - x_c), FP64 (rows of an odd number of
-// cells): the face difference is taken
+// cells, iterates of unaligned pairs): the face difference is taken
 // before the product, which keeps the residual accurate to rounding of the
 // differences when x is smooth or carries a large constant.
 __device__ __forceinline__ double flux64(const OuterView &O, const double *__restrict__ x, int i,
@@ -175,7 +193,7 @@ __device__ __forceinline__ double flux64(const OuterView &O, const double *__res
 }
 
 // The cells of this block's row tiles, one at a time: f(c, i, j, k) (rows of an
-// odd number of cells).
+// odd number of cells, iterates of unaligned pairs).
 template <class F>
 __device__ __forceinline__ void for_cells(const OuterView &O, int lb, F &&f)
 {

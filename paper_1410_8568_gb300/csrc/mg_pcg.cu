@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(kThreads) k_pcg_update(const OuterView *__rest
     if (!s->active) return;
     const int lb = blockIdx.x - start[e];
     const double a = s->alpha;
+    const bool pairs = p_pairs(O);
     Te *rv = (Te *)O.r;
     double v[1] = {0.0};
     struct In {
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(kThreads) k_pcg_update(const OuterView *__rest
     for_pairs(
         O, lb,
         [&](int c, bool both) {
-            if (both) return In{ld2(O.p + c), ld2(O.d + c), ld2(O.r64 + c), ld2(O.q + c)};
+            if (both) return In{ld_p(O, c, pairs), ld2(O.d + c), ld2(O.r64 + c), ld2(O.q + c)};
             const double2 z = make_double2(0.0, 0.0);
             In x{z, z, z, z};
             x.p.x = O.p[c];
