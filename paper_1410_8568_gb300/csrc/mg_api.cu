@@ -1210,6 +1210,17 @@ int gbmg::handle_alloc(const mg_grid *grid, const mg_params *params, void *strea
         v.G = h->G;
         v.err = h->err + 1;
     }
+    // the kernels that need attributes on this device
+    e = cudaSuccess;
+    if (h->mixed) e = march_opt_in();
+    if (e == cudaSuccess && first_tail_level(h) < h->L) e = tail_opt_in();
+    if (e == cudaSuccess) e = h->gmres ? coarse_gmres_opt_in() : coarse_setup_opt_in((int)h->lev[h->L - 1].N);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        note_cuda_error(e);
+        mg_destroy(h);
+        return MG_ECUDA;
+    }
     rc = tune_handle(h);
     if (rc) {
         mg_destroy(h);

@@ -273,26 +273,47 @@ void launch_coarse_solve(const CoarseView *cv, int count, int most, int cyc, con
              ov);
 }
 
+// 16 blocks per cluster are beyond the portable 8: the kernel opts in.
+template <int EP>
+static cudaError_t setup_opt_in()
+{
+    static DeviceOnce once;
+    return once([] {
+        return cudaFuncSetAttribute(k_coarse_setup<kSetupCluster, EP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    });
+}
+
 template <int EP>
 static void setup_cluster(const CoarseView &v, double inv_n2, cudaStream_t s)
 {
-    // 16 blocks per cluster are beyond the portable 8: the kernel opts in, once
-    static const cudaError_t opt_in =
-        cudaFuncSetAttribute(k_coarse_setup<kSetupCluster, EP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    (void)opt_in;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kSetupCluster;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(kSetupCluster);
-    c.blockDim = dim3(kSetupThreads);
-    c.stream = s;
-    c.attrs = at;
-    c.numAttrs = tl_dep_launch ? 2u : 1u;
-    cudaLaunchKernelEx(&c, k_coarse_setup<kSetupCluster, EP>, v, inv_n2);
+    if (setup_opt_in<EP>() != cudaSuccess) return;
+    ClusterLaunch l(kSetupCluster, kSetupCluster, kSetupThreads, 0, s);
+    cudaLaunchKernelEx(&l.c, k_coarse_setup<kSetupCluster, EP>, v, inv_n2);
+}
+
+template <int EP>
+static cudaError_t setup_supported()
+{
+    const cudaError_t e = setup_opt_in<EP>();
+    if (e != cudaSuccess) return e;
+    static DeviceOnce once;
+    return once([] {
+        ClusterLaunch l(kSetupCluster, kSetupCluster, kSetupThreads, 0, nullptr);
+        return l.placeable(k_coarse_setup<kSetupCluster, EP>);
+    });
+}
+
+// elements of a lane of the cluster for a coarsest grid of n cells (0: one block)
+static int setup_elements(int n)
+{
+    const int total = n * (n + 1) / 2;
+    return total <= kSetupThreads ? 0 : total <= 5 * kSetupCluster * kSetupThreads ? 5 : 17;
+}
+
+cudaError_t coarse_setup_opt_in(int n)
+{
+    const int ep = setup_elements(n);
+    return ep == 0 ? cudaSuccess : ep == 5 ? setup_supported<5>() : setup_supported<17>();
 }
 
 // One element per thread as long as one block holds them (n <= 31): without the
@@ -303,8 +324,9 @@ void launch_coarse_setup(const CoarseView &v, cudaStream_t s)
     const double inv_n2 = 1.0 / ((double)n * n);
     static_assert(kMaxCoarse <= kSetupThreads, "a thread per entry of a gathered column");
     static_assert(kMaxCoarse * (kMaxCoarse + 1) / 2 <= 17 * kSetupCluster * kSetupThreads, "elements in registers");
-    if (total <= kSetupThreads) launch_k(k_coarse_setup<1, 1>, 1, (total + 31) & ~31, 0, s, v, inv_n2);
-    else if (total <= 5 * kSetupCluster * kSetupThreads) setup_cluster<5>(v, inv_n2, s);
+    const int ep = setup_elements(n);
+    if (ep == 0) launch_k(k_coarse_setup<1, 1>, 1, (total + 31) & ~31, 0, s, v, inv_n2);
+    else if (ep == 5) setup_cluster<5>(v, inv_n2, s);
     else setup_cluster<17>(v, inv_n2, s);
 }
 

@@ -269,11 +269,11 @@ void launch_sweep_b(const Table &tb, int dir, double omega, int flags, const Out
     // the ring: 3 planes of at most B / nq + ... rows; (fR + 2) nq <= B, so
     // 3 (fR + 2) nx <= 12 B elements
     const size_t smem = (size_t)12 * B * sizeof(T);
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_sweep<T, B, MAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
-    }
+    static DeviceOnce once;
+    if (once([smem] {
+            return cudaFuncSetAttribute(k_sweep<T, B, MAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        }) != cudaSuccess)
+        return;
     const int single = table_single(tb);
     launch_k(k_sweep<T, B, MAYOUT>, tb.blocks, B, smem, s, tb.lv, tb.start, tb.count, dir, (T)omega, flags,
              tb.cyc, ov, table_view(tb), single);

@@ -271,40 +271,44 @@ __global__ void __launch_bounds__(kGmThreads, 1) k_coarse_gmres(const CoarseView
     cluster_sync();  // no block leaves while another may still write its sums
 }
 
-namespace {
-
-// 16 blocks per cluster are beyond the portable 8: the kernel opts in, once.
+// 16 blocks per cluster are beyond the portable 8: the kernel opts in.
 template <class T>
-void gm_opt_in()
+static cudaError_t gm_opt_in()
 {
-    static const cudaError_t done = [] {
-        cudaFuncSetAttribute(k_coarse_gmres<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGmSmem);
+    static DeviceOnce once;
+    return once([] {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_coarse_gmres<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGmSmem);
+        if (e != cudaSuccess) return e;
         return cudaFuncSetAttribute(k_coarse_gmres<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    }();
-    (void)done;
+    });
 }
-
-}  // namespace
 
 template <class T>
 void launch_coarse_gmres(const CoarseView *cv, int count, int cyc, const OuterView *ov, cudaStream_t s)
 {
-    const int size = kGmCluster;
-    gm_opt_in<T>();
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)size;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3((unsigned)(count * size));
-    c.blockDim = dim3(kGmThreads);
-    c.dynamicSmemBytes = kGmSmem;
-    c.stream = s;
-    c.attrs = at;
-    c.numAttrs = tl_dep_launch ? 2u : 1u;
-    cudaLaunchKernelEx(&c, k_coarse_gmres<T>, cv, cyc, ov, size);
+    if (gm_opt_in<T>() != cudaSuccess) return;
+    ClusterLaunch l(kGmCluster, count * kGmCluster, kGmThreads, kGmSmem, s);
+    cudaLaunchKernelEx(&l.c, k_coarse_gmres<T>, cv, cyc, ov, kGmCluster);
+}
+
+template <class T>
+static cudaError_t gm_supported()
+{
+    const cudaError_t e = gm_opt_in<T>();
+    if (e != cudaSuccess) return e;
+    static DeviceOnce once;
+    return once([] {
+        ClusterLaunch l(kGmCluster, kGmCluster, kGmThreads, kGmSmem, nullptr);
+        return l.placeable(k_coarse_gmres<T>);
+    });
+}
+
+// (a mixed handle solves its coarsest grid in FP64 on request: mg_coarse_solve)
+cudaError_t coarse_gmres_opt_in()
+{
+    const cudaError_t e = gm_supported<float>();
+    return e != cudaSuccess ? e : gm_supported<double>();
 }
 
 template void launch_coarse_gmres<float>(const CoarseView *, int, int, const OuterView *, cudaStream_t);

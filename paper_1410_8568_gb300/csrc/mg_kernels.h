@@ -135,6 +135,13 @@ bool staged_fits(const int n[3], int per);
 int march_chunk(const int n[3], int per);
 int march_layout(LevelView &v, int kc);
 void launch_march(const Table &, int dir, double omega, int flags, const OuterView *ov, cudaStream_t);
+// attributes of the kernels that need them, on the current device (each launch
+// sees to its own; here so that mg_create can report a device that refuses them;
+// n: cells of the coarsest grid)
+cudaError_t march_opt_in();
+cudaError_t tail_opt_in();
+cudaError_t coarse_setup_opt_in(int n);
+cudaError_t coarse_gmres_opt_in();
 // V-cycle stages below the row-tiled levels; cyc as Table::cyc
 // (the tail: FP32 cycles, mg_tail.cu; tail_floats: shared-memory elements of its
 // level t of nt with N cells)

@@ -23,6 +23,8 @@
 
 #include <utility>
 
+#include "mg_optin.h"
+
 namespace gbmg {
 
 __device__ __forceinline__ void dep_entry()
@@ -62,6 +64,37 @@ inline void launch_k(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, c
     c.numAttrs = tl_dep_launch ? 1u : 0u;
     cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
 }
+
+// Launch of clusters of `size` blocks, with the attribute when enabled.
+struct ClusterLaunch {
+    cudaLaunchAttribute at[2];
+    cudaLaunchConfig_t c = {};
+    ClusterLaunch(int size, int blocks, int threads, size_t smem, cudaStream_t s)
+    {
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)size;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
+        c.gridDim = dim3((unsigned)blocks);
+        c.blockDim = dim3((unsigned)threads);
+        c.dynamicSmemBytes = smem;
+        c.stream = s;
+        c.attrs = at;
+        c.numAttrs = tl_dep_launch ? 2u : 1u;
+    }
+    ClusterLaunch(const ClusterLaunch &) = delete;
+    ClusterLaunch &operator=(const ClusterLaunch &) = delete;
+    // whether the current device can hold such a cluster at all
+    template <class K>
+    cudaError_t placeable(K *kernel)
+    {
+        c.numAttrs = 1;
+        int clusters = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &c);
+        return e != cudaSuccess ? e : clusters > 0 ? cudaSuccess : cudaErrorLaunchOutOfResources;
+    }
+};
 
 // Process default for plans: on unless the environment sets MG_DEP_LAUNCH=0.
 int dep_launch_default();

@@ -510,12 +510,16 @@ int march_layout(LevelView &v, int kc)
     return v.fS * ((nz + v.fKc - 1) / v.fKc);
 }
 
+cudaError_t march_opt_in()
+{
+    static DeviceOnce once;
+    return once(
+        [] { return cudaFuncSetAttribute(k_march, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(March)); });
+}
+
 void launch_march(const Table &tb, int dir, double omega, int flags, const OuterView *ov, cudaStream_t s)
 {
-    if (tb.blocks == 0) return;
-    static const cudaError_t opt_in =
-        cudaFuncSetAttribute(k_march, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(March));
-    (void)opt_in;
+    if (tb.blocks == 0 || march_opt_in() != cudaSuccess) return;
     launch_k(k_march, tb.blocks, 32 * W, sizeof(March), s, tb.lv, tb.start, tb.count, dir, (float)omega, flags, tb.cyc,
              table_view(tb), table_single(tb));
     if (flags & kOuter)

@@ -562,13 +562,17 @@ int tail_floats(int N, int t, int nt, bool flux)
     return 2 * half_pad(N, t) + N + (t > 0 ? N + N + 3 * N + kItemWords * (N / 2) + (flux ? N : 0) : 0);
 }
 
+// More than 48 KB of shared memory: a 16^3 first level takes 32 KB, the levels
+// below it about 45 KB more.
+cudaError_t tail_opt_in()
+{
+    static DeviceOnce once;
+    return once([] { return cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmemMax); });
+}
+
 void launch_tail(const TailView *tv, int count, size_t smem, double omega, int nu1, int nu2, int cyc, cudaStream_t s)
 {
-    // opt in to more than 48 KB of shared memory, once: a 16^3 first level takes
-    // 32 KB, the levels below it about 45 KB more
-    static const cudaError_t opt_in =
-        cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmemMax);
-    (void)opt_in;
+    if (tail_opt_in() != cudaSuccess) return;
     launch_k(k_tail, count, kTailThreads, smem, s, tv, (float)omega, nu1, nu2, cyc);
 }
 
