@@ -912,10 +912,12 @@ static int run_plan_t(Plan &P, Prof &pf, bool use_graph)
 
 void plan_bind(Plan &P, int g, const double *rhs, double *p, double tol, int max_iters)
 {
-    P.ov_h[g].b = rhs;
-    P.ov_h[g].p = p;
-    P.ov_h[g].tol = tol;
-    P.ov_h[g].max_iters = max_iters;
+    OuterView &v = P.ov_h[g];
+    v.b = rhs;
+    v.p = p;
+    v.tol = tol;
+    v.max_iters = max_iters;
+    v.mitems = ((uintptr_t)p & 15) == 0 ? v.mall : 0;  // (kernels that march p load pairs of it)
 }
 
 int plan_upload(Plan &P)
@@ -997,10 +999,7 @@ int run_plan(Plan &P, Prof &pf, const double *const *rhs, double *const *p, cons
     for (int g = 0; g < P.G; g++) {
         if (!rhs[g] || !p[g] || !(tol[g] >= 0.0)) return MG_EINVAL;
         if (((uintptr_t)p[g] & 15) != 0) return MG_EINVAL;  // (the documented alignment)
-        P.ov_h[g].b = rhs[g];
-        P.ov_h[g].p = p[g];
-        P.ov_h[g].tol = tol[g];
-        P.ov_h[g].max_iters = P.hs[g]->prm.max_iters;
+        plan_bind(P, g, rhs[g], p[g], tol[g], P.hs[g]->prm.max_iters);
     }
     const bool use_graph = P.prm.use_graph != 0;
     int rc = P.mixed ? run_plan_t<float>(P, pf, use_graph) : run_plan_t<double>(P, pf, use_graph);

@@ -218,8 +218,9 @@ struct OuterView {
     FastDiv dxt;         // division by the row tiles of a row, fine_xtiles(n[0])
     // march_pairs: items, planes per piece, log2 of a block's z pieces, tiles of
     // pairs per plane; division by them and by the pairs of a row (0 items: rows of
-    // an odd number of cells)
+    // an odd number of cells); items as if p were made of aligned pairs (host)
     int mitems, mkz, msub, mtiles;
+    int mall;
     FastDiv mdt, mdx;
     float *xp3[3];
     float *xb[2];
@@ -323,6 +324,7 @@ inline void outer_march(OuterView &v)
             }
         }
     }
+    v.mall = v.mitems;
     v.mdt = make_fastdiv((unsigned)v.mtiles);
     v.mdx = make_fastdiv(v.n[0] >= 2 ? (unsigned)(v.n[0] / 2) : 1u);
 }

@@ -1097,7 +1097,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_residual(const OuterView *__res
                     racc += r1 * r1;
                 }
             });
-    } else if (O.mitems && p_pairs(O)) {
+    } else if (O.mitems) {  // (0 also where p is not made of aligned pairs)
         march_pairs(
             O, O.p, lb,
             [&](int c) {

@@ -29,11 +29,15 @@ def test_pairs_of_the_callers_iterate_move_behind_the_alignment_test():
         for m in re.finditer(r"\(double2 \*\)po\.p", src):
             body = src[src.rfind("outer_out(", 0, m.start()):m.start()]
             assert "(size_t)po.p & 15" in body, path
+        # the march over p runs where there are items, and an unaligned p has none
         for m in re.finditer(r"march_pairs\(\s*O, O\.p\b", src):
-            cond = src[src.rfind("if (", 0, m.start()):m.start()]
-            assert "p_pairs(O)" in cond, path
+            assert "O.mitems" in src[src.rfind("if (", 0, m.start()):m.start()], path
             marches += 1
     assert helpers == 2 and marches == 1
+    api = open(os.path.join(CSRC, "mg_api.cu")).read()
+    assert len(re.findall(r"\bmitems\b", api)) == 1
+    assert re.search(r"mitems = \(\(uintptr_t\)p & 15\) == 0 \? v\.mall : 0;", api)
+    assert len(re.findall(r"\bv\.p = p;", api)) == 1 and "ov_h[g].p" not in api, "p is bound in one place"
 
 
 def problem(shape, seed):
