@@ -486,6 +486,7 @@ int Plan::fill(mg_handle *const *handles, int count)
         v.part = h->part;
         v.nblk = h->nblk0;
         v.st = h->state;
+        v.tiny = h->err + 3;
         v.tol = 1e-10;
         v.max_iters = h->prm.max_iters;
         v.inner = prm.inner_cycles;
@@ -1037,6 +1038,7 @@ static int upload_faces(mg_handle *h)
             a.wc[d] = h->lev[l].w64[d];
             a.wc32[d] = h->mixed ? h->lev[l].w32[d] : nullptr;
         }
+        a.tiny = h->err + 3;
         a.dx = make_fastdiv((unsigned)a.nc[0]);
         a.dy = make_fastdiv((unsigned)a.nc[1]);
         launch_coarsen_faces(a, h->stream);
@@ -1079,7 +1081,7 @@ int gbmg::set_faces_impl(mg_handle *h, const double *ax, const double *ay, const
 {
     DepScope dep(dep_launch_default());
     if (!ax || !ay || !az) return MG_EINVAL;
-    CK(cudaMemsetAsync(h->err, 0, 3 * sizeof(int), h->stream));
+    CK(cudaMemsetAsync(h->err, 0, 4 * sizeof(int), h->stream));
     FaceArgs a;
     memset(&a, 0, sizeof(a));
     const double *in[3] = {ax, ay, az};
@@ -1093,6 +1095,7 @@ int gbmg::set_faces_impl(mg_handle *h, const double *ax, const double *ay, const
     }
     a.per = h->per;
     a.err = h->err;
+    a.tiny = h->err + 3;
     launch_scale_faces(a, h->stream);
     return upload_faces(h);
 }
@@ -1101,7 +1104,7 @@ static int set_density_impl(mg_handle *h, const double *rho, int mode)
 {
     DepScope dep(dep_launch_default());
     if (!rho || (mode != MG_FACE_HARMONIC && mode != MG_FACE_ARITHMETIC)) return MG_EINVAL;
-    CK(cudaMemsetAsync(h->err, 0, 3 * sizeof(int), h->stream));
+    CK(cudaMemsetAsync(h->err, 0, 4 * sizeof(int), h->stream));
     FaceArgs a;
     memset(&a, 0, sizeof(a));
     for (int d = 0; d < 3; d++) {
@@ -1115,6 +1118,7 @@ static int set_density_impl(mg_handle *h, const double *rho, int mode)
     a.mode = mode;
     a.rho = rho;
     a.err = h->err;
+    a.tiny = h->err + 3;
     launch_faces_from_density(a, h->stream);
     return upload_faces(h);
 }
@@ -1651,6 +1655,7 @@ static int unit_view(mg_handle *h, int level, int prec, const void *x, void *b,
     const int var = (tiles != kFineTiles && level + 1 < h->L) ? h->tile[kind][level] : 0;
     const int blocks = tiles == kFineTiles ? fine_blocks(v.n) : kernel_blocks(kind, v.n, v.nc, var);
     const int starts[2] = {0, blocks};
+    CK(cudaMemcpyAsync(&h->dstate->tiny, h->err + 3, sizeof(int), cudaMemcpyDeviceToDevice, h->stream));
     CK(cudaMemcpyAsync(h->dview, &v, sizeof(v), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemcpyAsync(h->dstart, starts, sizeof(starts), cudaMemcpyHostToDevice, h->stream));
     *tb = Table{h->dview, h->dstart, 1, blocks, var,
@@ -1716,6 +1721,7 @@ int mg_smooth_onepass(mg_handle *h, int level, int prec, const void *b, void *x,
     fill_fastdiv(v);
     const int blocks = kc ? march_layout(v, kc) : sweep_layout(v, variant);
     const int starts[2] = {0, blocks};
+    CK(cudaMemcpyAsync(&h->dstate->tiny, h->err + 3, sizeof(int), cudaMemcpyDeviceToDevice, h->stream));
     CK(cudaMemcpyAsync(h->dview, &v, sizeof(v), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemcpyAsync(h->dstart, starts, sizeof(starts), cudaMemcpyHostToDevice, h->stream));
     Table tb{h->dview, h->dstart, 1, blocks, variant};

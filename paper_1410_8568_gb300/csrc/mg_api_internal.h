@@ -76,7 +76,8 @@ struct mg_handle {
     double *b0 = nullptr;      // right-hand side minus its mean (FP64)
     double *part = nullptr;    // reduction partials of the outer launches
     int nblk0 = 0;
-    int *err = nullptr;        // [0] bad coefficient, [1] singular coarsest grid, [2] device wait gave up
+    int *err = nullptr;        // [0] bad coefficient, [1] singular coarsest grid, [2] device wait gave up;
+                               // [3] not an error: some FP32 face is subnormal
     gbmg::GridState *state = nullptr;    // solve state of this grid (kept across plans)
     gbmg::GridState *dstate = nullptr;   // always-active state of the unit calls
     gbmg::LevelView *dview = nullptr;    // view slot of the unit calls

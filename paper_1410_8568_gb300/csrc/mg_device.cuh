@@ -40,6 +40,7 @@ struct GridState {
     int cycles_next;  // V-cycles of the next refinement step (1 .. inner)
     int steps;        // refinement steps done
     int pnz;          // the caller's starting iterate has a nonzero cell (multigrid iteration)
+    int tiny;         // some FP32 face of the handle is subnormal (see tiny_scale)
     double rprev;     // ||r|| before the last refinement step
     double rz;      // conjugate gradients: r . z of the current step
     double alpha;   //   step length
@@ -201,6 +202,7 @@ struct OuterView {
     double *part;        // kPart doubles per block of this grid's outer launches
     int nblk;            // blocks of this grid in an outer launch
     GridState *st;
+    const int *tiny;     // the handle's flag of subnormal FP32 faces, for the state
     double tol;
     int max_iters;
     int inner;           // V-cycles per refinement step

@@ -33,8 +33,8 @@ template <class T>
 __device__ __forceinline__ Quad<T> relax_quad_global(const T *__restrict__ x, const T *__restrict__ b,
                                                      const T *__restrict__ wx, const T *__restrict__ wy,
                                                      const T *__restrict__ wz, int nx, int ny, int nz, int per,
-                                                     int j, int k, int qx, int colour, T omega, bool zero,
-                                                     const T *__restrict__ dinv)
+                                                     int j, int k, int qx, int colour, T omega, T tiny,
+                                                     bool zero, const T *__restrict__ dinv)
 {
     const int sy = nx, sz = nx * ny;
     const int i0 = qx << 2;
@@ -92,8 +92,8 @@ __device__ __forceinline__ Quad<T> relax_quad_global(const T *__restrict__ x, co
         v0 = relax_cell_inv(xc0, xl0, xr0, fl0, fr0, fs0, fn0, fb0, ft0, xs0, xn0, xb0, xt0, b0, omega, di0);
         v1 = relax_cell_inv(xc1, xl1, xr1, fl1, fr1, fs1, fn1, fb1, ft1, xs1, xn1, xb1, xt1, b1, omega, di1);
     } else {
-        v0 = relax_cell(xc0, xl0, xr0, fl0, fr0, fs0, fn0, fb0, ft0, xs0, xn0, xb0, xt0, b0, omega);
-        v1 = relax_cell(xc1, xl1, xr1, fl1, fr1, fs1, fn1, fb1, ft1, xs1, xn1, xb1, xt1, b1, omega);
+        v0 = relax_cell(xc0, xl0, xr0, fl0, fr0, fs0, fn0, fb0, ft0, xs0, xn0, xb0, xt0, b0, omega, tiny);
+        v1 = relax_cell(xc1, xl1, xr1, fl1, fr1, fs1, fn1, fb1, ft1, xs1, xn1, xb1, xt1, b1, omega, tiny);
     }
     Quad<T> out = xq;
     out.v[0] = par ? xq.v[0] : v0;
@@ -113,7 +113,7 @@ __device__ __forceinline__ Quad<T> black_quad(const Quad<T> &xq, const T *orow, 
                                               const Quad<T> &xbq, const Quad<T> &xtq, const T *__restrict__ b,
                                               const T *__restrict__ wx, const T *__restrict__ wy,
                                               const T *__restrict__ wz, int nx, int ny, int nz, int per, int j,
-                                              int k, int qx, T omega, const T *__restrict__ dinv)
+                                              int k, int qx, T omega, T tiny, const T *__restrict__ dinv)
 {
     const int sy = nx, sz = nx * ny;
     const int i0 = qx << 2;
@@ -151,8 +151,8 @@ __device__ __forceinline__ Quad<T> black_quad(const Quad<T> &xq, const T *orow, 
         v0 = relax_cell_inv(xc0, xl0, xr0, fl0, fr0, fs0, fn0, fb0, ft0, xs0, xn0, xb0, xt0, b0, omega, di0);
         v1 = relax_cell_inv(xc1, xl1, xr1, fl1, fr1, fs1, fn1, fb1, ft1, xs1, xn1, xb1, xt1, b1, omega, di1);
     } else {
-        v0 = relax_cell(xc0, xl0, xr0, fl0, fr0, fs0, fn0, fb0, ft0, xs0, xn0, xb0, xt0, b0, omega);
-        v1 = relax_cell(xc1, xl1, xr1, fl1, fr1, fs1, fn1, fb1, ft1, xs1, xn1, xb1, xt1, b1, omega);
+        v0 = relax_cell(xc0, xl0, xr0, fl0, fr0, fs0, fn0, fb0, ft0, xs0, xn0, xb0, xt0, b0, omega, tiny);
+        v1 = relax_cell(xc1, xl1, xr1, fl1, fr1, fs1, fn1, fb1, ft1, xs1, xn1, xb1, xt1, b1, omega, tiny);
     }
     Quad<T> out = xq;
     out.v[0] = par ? xq.v[0] : v0;
@@ -166,7 +166,7 @@ __device__ __forceinline__ Quad<T> black_quad(const Quad<T> &xq, const T *orow, 
 // lb / fS of fKc planes.  B threads: thread t relaxes quad t % nq of slot row
 // t / nq, slot 0 being the row below the strip and slot fR + 1 the row above.
 template <class T, int B, bool OUT>
-__device__ __forceinline__ void sweep_body(const LevelView &L, int lb, int dir, T omega, bool zero,
+__device__ __forceinline__ void sweep_body(const LevelView &L, int lb, int dir, T omega, T tiny, bool zero,
                                            const OuterOut &po, T *sm)
 {
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2], per = L.per, nq = nx >> 2;
@@ -209,7 +209,7 @@ __device__ __forceinline__ void sweep_body(const LevelView &L, int lb, int dir, 
             else vpl = false;
         }
         if (vrow && vpl) {
-            q0 = relax_quad_global<T>(xin, b, wx, wy, wz, nx, ny, nz, per, jj, kk, tq, 0, omega, zero, dinv);
+            q0 = relax_quad_global<T>(xin, b, wx, wy, wz, nx, ny, nz, per, jj, kk, tq, 0, omega, tiny, zero, dinv);
             stq(sm + rk * rowlen + tr * nx + (tq << 2), q0);
         }
         __syncthreads();
@@ -218,7 +218,8 @@ __device__ __forceinline__ void sweep_body(const LevelView &L, int lb, int dir, 
             const int rp = rk == 0 ? 2 : rk - 1;  // ring slot of plane k - 1
             const T *plane = sm + rp * rowlen;
             const Quad<T> out = black_quad<T>(q1, plane + tr * nx, plane + (tr - 1) * nx, plane + (tr + 1) * nx,
-                                              q2, q0, b, wx, wy, wz, nx, ny, nz, per, j, kb, tq, omega, dinv);
+                                              q2, q0, b, wx, wy, wz, nx, ny, nz, per, j, kb, tq, omega, tiny,
+                                              dinv);
             const int c = (j + ny * kb) * nx + (tq << 2);
             stq(xout + c, out);
             if constexpr (OUT) add_outer_quad<T>(po, c, out.v, 0xF);
@@ -235,15 +236,20 @@ __device__ __forceinline__ void sweep_entry(const LevelView &L, int lb, int dir,
 {
     // the whole block returns together (a grid's state is uniform), so the
     // barriers inside the body see every thread
+    T tiny = T(1);
+    if constexpr (sizeof(T) == 4) {
+        tiny = tiny_scale(L.st);
+        omega *= tiny;
+    }
     if (!in_cycle(L.st, cyc)) return;
     const bool zero = flags & kZeroGuess;
     if constexpr (MAYOUT) {
         if (last_cycle(L.st, cyc)) {
-            sweep_body<T, B, true>(L, lb, dir, omega, zero, outer_out(ov[L.g]), sm);
+            sweep_body<T, B, true>(L, lb, dir, omega, tiny, zero, outer_out(ov[L.g]), sm);
             return;
         }
     }
-    sweep_body<T, B, false>(L, lb, dir, omega, zero, OuterOut{}, sm);
+    sweep_body<T, B, false>(L, lb, dir, omega, tiny, zero, OuterOut{}, sm);
 }
 
 template <class T, int B, bool MAYOUT>

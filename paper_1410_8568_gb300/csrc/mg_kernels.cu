@@ -120,7 +120,7 @@ struct LoadPlain {
 // a row (one 16-byte vector per operand for FP32, two for FP64), relaxes the 2
 // cells of the launch's colour and writes the other two back unchanged;
 // otherwise (small coarse levels) one cell per thread.  The FP32 cycle uses a
-// 2-ulp division (relax_div): the inner cycle is a preconditioner and only
+// 2-ulp division (relax_quot): the inner cycle is a preconditioner and only
 // steers convergence; the FP64 path divides exactly.
 //
 // flags: kZeroGuess  (red launch) the iterate is zero on entry: red cells get
@@ -165,14 +165,14 @@ __device__ __forceinline__ void half_body(const LevelView &L, int lb, int colour
                     v = di[c] > T(0) ? omega * ((-b[c]) * di[c]) : T(0);
                 } else {
                     const T d = diag_of(wx, wy, wz, nx, ny, nz, per, i, t.j, t.k, c);
-                    v = relaxable(d) ? omega * relax_div(-b[c], d) : T(0);
+                    v = omega * relax_quot(-b[c], d);
                 }
             } else {
                 const T xc = x[c];
                 T d, f;
                 stencil(wx, wy, wz, LoadPlain<T>{x}, nx, ny, nz, per, i, t.j, t.k, c, xc, d, f);
                 if (di) v = di[c] > T(0) ? xc + omega * ((f - b[c]) * di[c]) : xc;  // (rows of other than whole quads)
-                else v = relaxable(d) ? xc + omega * relax_div(f - b[c], d) : xc;
+                else v = xc + omega * relax_quot(f - b[c], d);
             }
             x[c] = v;
             if constexpr (OUT) add_outer<T>(po, (int)c, v);
@@ -445,7 +445,8 @@ __global__ void __launch_bounds__(kThreads) k_apply(const LevelView *__restrict_
 //   widen_pos:   exact float -> double (normal positive f).
 //   trunc_pos:   double -> float, low 29 mantissa bits dropped (a seed).
 //   narrow_rn:   double -> float, round to nearest, ties to even; values
-//                outside the fast range take the hardware conversion.
+//                outside the fast range take the hardware conversion, and set
+//                *tiny (if given) when they give a subnormal.
 __device__ __forceinline__ double widen_pos(float f)
 {
     const unsigned b = __float_as_uint(f);
@@ -455,12 +456,16 @@ __device__ __forceinline__ float trunc_pos(unsigned hi, unsigned lo)
 {
     return __uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29));
 }
-__device__ __forceinline__ float narrow_rn(double d)
+__device__ __forceinline__ float narrow_rn(double d, int *tiny = nullptr)
 {
     const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
     // positive, biased exponent 897 .. 1150: a normal float (or, rounding up
     // from the largest, the overflow to infinity that the rounding rule gives)
-    if ((hi >> 20) - 897u > 253u) return (float)d;
+    if ((hi >> 20) - 897u > 253u) {
+        const float f = (float)d;
+        if (tiny && f > 0.f && f < kTinyDiag) *tiny = 1;
+        return f;
+    }
     unsigned b = __float_as_uint(trunc_pos(hi, lo));
     const unsigned rem = lo & 0x1FFFFFFFu, half = 0x10000000u;
     b += (rem > half || (rem == half && (b & 1u))) ? 1u : 0u;  // a carry steps the exponent
@@ -551,7 +556,7 @@ __global__ void __launch_bounds__(kThreads) k_faces_from_density(const __grid_co
                 else v = (0.5 * a.scale[d]) * (recip(rho_l) + inv_c);
             }
             if (a.out64[d]) a.out64[d][c] = v;
-            if (a.out32[d]) a.out32[d][c] = narrow_rn(v);
+            if (a.out32[d]) a.out32[d][c] = narrow_rn(v, a.tiny);
             if (a.out32lo[d]) a.out32lo[d][c] = (float)(v - (double)(float)v);
         }
         if (!ok && a.err) *a.err = 1;
@@ -576,7 +581,7 @@ __global__ void __launch_bounds__(kThreads) k_scale_faces(FaceArgs a)
                 v = alpha * a.scale[d];
             }
             a.out64[d][c] = v;
-            if (a.out32[d]) a.out32[d][c] = narrow_rn(v);
+            if (a.out32[d]) a.out32[d][c] = narrow_rn(v, a.tiny);
             if (a.out32lo[d]) a.out32lo[d][c] = (float)(v - (double)(float)v);
         }
     }
@@ -713,7 +718,7 @@ __global__ void __launch_bounds__(kThreads) k_coarsen_faces(CoarsenArgs a)
                 }
             const double w = s * 0.0625;
             a.wc[d][C] = w;
-            if (a.wc32[d]) a.wc32[d][C] = narrow_rn(w);
+            if (a.wc32[d]) a.wc32[d][C] = narrow_rn(w, a.tiny);
         }
     }
 }
@@ -745,6 +750,7 @@ __global__ void k_begin(const OuterView *__restrict__ ov)
     s->xinv = 1.0;
     s->rprev = 0.0;
     s->pnz = 0;
+    s->tiny = *O.tiny;
 }
 
 // Partial sums of the caller's right-hand side (which = 0, partial slot 3) or

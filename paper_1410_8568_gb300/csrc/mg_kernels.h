@@ -39,6 +39,7 @@ struct FaceArgs {
     double scale[3];         // 1 for raw alpha, 1/h_d^2 for level-0 coefficients
     double *out64[3];
     float *out32[3];         // optional FP32 copy (round to nearest)
+    int *tiny;               // optional: set when a face of that copy is subnormal
     float *out32lo[3];       // optional: out64 - out32 rounded to FP32 (float-pair faces)
     FastDiv dx, dy;          // division by n[0], n[1] (set by the launcher)
     int *err;                // set to 1 on a non-positive / non-finite value
@@ -83,6 +84,7 @@ struct CoarsenArgs {
     const double *wf[3];
     double *wc[3];
     float *wc32[3];
+    int *tiny;               // optional: set when an FP32 face is subnormal
     FastDiv dx, dy;  // division by nc[0] and by nc[1]
 };
 

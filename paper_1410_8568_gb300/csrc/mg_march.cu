@@ -78,19 +78,19 @@ __device__ __forceinline__ float2 pick(const float4 &q)
 
 // Relaxation of the cells PAR, PAR + 2 of a quad: c their values, o the two
 // other cells' values (offsets 1 - PAR, 3 - PAR), e the x neighbour outside
-// the quad (west of cell 0 if PAR = 0, east of cell 3 if PAR = 1).
+// the quad (west of cell 0 if PAR = 0, east of cell 3 if PAR = 1); omega, tiny: see relax_cell.
 template <int PAR>
 __device__ __forceinline__ float2 relax2(float2 c, float2 o, float e, const float4 &fx, float fe, float2 fs, float2 fn,
                                          float2 fb, float2 ft, float2 xs, float2 xn, float2 xb, float2 xt, float2 b,
-                                         float omega)
+                                         float omega, float tiny)
 {
     float2 v;
     if (PAR == 0) {
-        v.x = relax_cell(c.x, e, o.x, fx.x, fx.y, fs.x, fn.x, fb.x, ft.x, xs.x, xn.x, xb.x, xt.x, b.x, omega);
-        v.y = relax_cell(c.y, o.x, o.y, fx.z, fx.w, fs.y, fn.y, fb.y, ft.y, xs.y, xn.y, xb.y, xt.y, b.y, omega);
+        v.x = relax_cell(c.x, e, o.x, fx.x, fx.y, fs.x, fn.x, fb.x, ft.x, xs.x, xn.x, xb.x, xt.x, b.x, omega, tiny);
+        v.y = relax_cell(c.y, o.x, o.y, fx.z, fx.w, fs.y, fn.y, fb.y, ft.y, xs.y, xn.y, xb.y, xt.y, b.y, omega, tiny);
     } else {
-        v.x = relax_cell(c.x, o.x, o.y, fx.y, fx.z, fs.x, fn.x, fb.x, ft.x, xs.x, xn.x, xb.x, xt.x, b.x, omega);
-        v.y = relax_cell(c.y, o.y, e, fx.w, fe, fs.y, fn.y, fb.y, ft.y, xs.y, xn.y, xb.y, xt.y, b.y, omega);
+        v.x = relax_cell(c.x, o.x, o.y, fx.y, fx.z, fs.x, fn.x, fb.x, ft.x, xs.x, xn.x, xb.x, xt.x, b.x, omega, tiny);
+        v.y = relax_cell(c.y, o.y, e, fx.w, fe, fs.y, fn.y, fb.y, ft.y, xs.y, xn.y, xb.y, xt.y, b.y, omega, tiny);
     }
     return v;
 }
@@ -136,7 +136,7 @@ __device__ __forceinline__ void copy16(unsigned dst, const float *src)
 // the same parity (same values to the same places); only the stores of own
 // cells are guarded.
 template <bool ZERO>
-__device__ __forceinline__ void march_body(const LevelView &L, int lb, int dir, float omega, March &sh)
+__device__ __forceinline__ void march_body(const LevelView &L, int lb, int dir, float omega, float tiny, March &sh)
 {
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
     const float *__restrict__ xin = (const float *)(dir ? L.x2 : L.x);
@@ -275,13 +275,13 @@ __device__ __forceinline__ void march_body(const LevelView &L, int lb, int dir, 
             xn = pick<PAR>(sh.x[slot][me + 2 * tq]);
         }
         const float2 red = relax2<PAR>(pick<PAR>(xk), ob, xo, fx, fe, pick<PAR>(fs), pick<PAR>(fn), pick<PAR>(zk),
-                                       pick<PAR>(zp), xs, xn, xm, pick<PAR>(xp), pick<PAR>(b), omega);
+                                       pick<PAR>(zp), xs, xn, xm, pick<PAR>(xp), pick<PAR>(b), omega, tiny);
         // black of plane k - 1 (the red cell beyond the tile from the halo warp)
         float ro = PAR ? __shfl_sync(0xffffffffu, B.r.x, le) : __shfl_sync(0xffffffffu, B.r.y, lw);
         if (own && k > k0) {
             if (PAR ? ld_e : ld_w) ro = sh.halo[prv][r];
             const float2 v = relax2<PAR>(B.x, B.r, ro, B.fx, B.fe, B.fs, B.fn, B.fb, pick<PAR>(zk),
-                                         sh.red[prv][me - tq], sh.red[prv][me + tq], r2, red, B.b, omega);
+                                         sh.red[prv][me - tq], sh.red[prv][me + tq], r2, red, B.b, omega, tiny);
             const int c = cst;
             Quad<float> o;
             o.v[PAR] = v.x;
@@ -306,7 +306,7 @@ __device__ __forceinline__ void march_body(const LevelView &L, int lb, int dir, 
 #pragma unroll
             for (int u = 0; u < 14; u++) h[u] = ZERO && (u < 3 || (u > 8 && u < 13)) ? 0.f : sh.cell[slot][u][lane];
             sh.halo[cur][lane + 1] = relax_cell(h[0], h[1], h[2], h[3], h[4], h[5], h[6], h[7], h[8], h[9], h[10],
-                                                h[11], h[12], h[13], omega);
+                                                h[11], h[12], h[13], omega, tiny);
         }
         cst += sz;
         xm = ob;
@@ -347,10 +347,11 @@ __device__ __forceinline__ void march_entry(const LevelView &L, int lb, int dir,
 {
     extern __shared__ __align__(16) unsigned char march_smem[];
     March &sh = *(March *)march_smem;
+    const float tiny = tiny_scale(L.st);
     // the whole block returns together (a grid's state is uniform)
     if (!in_cycle(L.st, cyc)) return;
-    if (flags & kZeroGuess) march_body<true>(L, lb, dir, omega, sh);
-    else march_body<false>(L, lb, dir, omega, sh);
+    if (flags & kZeroGuess) march_body<true>(L, lb, dir, omega * tiny, tiny, sh);
+    else march_body<false>(L, lb, dir, omega * tiny, tiny, sh);
 }
 
 __global__ void __launch_bounds__(32 * W, 1) k_march(const LevelView *__restrict__ lv, const int *__restrict__ start,

@@ -63,28 +63,34 @@ __device__ __forceinline__ void stq(T *p, const Quad<T> &q)
     }
 }
 
-// num / den for a den in the normal range.  FP32 (inner cycles): the 1-ulp
-// reciprocal and a product, within 2 ulp of the quotient, two instructions;
-// the approximate division of the same accuracy also scales subnormal and huge
-// divisors, in eight, which the issue-bound sweeps feel.
+// num / d of a relaxation, d the cell's diagonal: 0 for a cell without faces
+// (d = 0), which keeps its value.  FP32 (inner cycles): the 1-ulp reciprocal and a
+// product, within 2 ulp of the quotient, two instructions; the approximate
+// division of the same accuracy scales every divisor, in eight, which the
+// issue-bound sweeps feel.  Subnormal diagonals, whose reciprocal the
+// approximation does not give, are scaled here alone, behind a branch.
+constexpr float kTinyDiag = 1.17549435e-38f;  // the smallest normal float
+constexpr float kTinyScale = 16777216.f;      // 2^24: every subnormal times it is normal
+__device__ __forceinline__ float rcp_ftz(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float tiny_quot(float num, float d)
+{
+    return d > 0.f ? num * rcp_ftz(d * kTinyScale) * kTinyScale : 0.f;
+}
 template <class T>
-__device__ __forceinline__ T relax_div(T num, T den)
+__device__ __forceinline__ T relax_quot(T num, T d)
 {
     if constexpr (sizeof(T) == 4) {
-        float r;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(den));
-        return num * r;
+        float q = num * rcp_ftz(d);
+        if (!(d >= kTinyDiag)) q = tiny_quot(num, d);
+        return q;
     } else {
-        return num / den;
+        return d > T(0) ? num / d : T(0);
     }
-}
-// a diagonal that a cell can be relaxed with: positive (FP32: and normal; cells
-// of a smaller one would carry corrections beyond the FP32 range)
-template <class T>
-__device__ __forceinline__ bool relaxable(T d)
-{
-    if constexpr (sizeof(T) == 4) return d >= 1.17549435e-38f;
-    else return d > T(0);
 }
 
 // half-sweep flags: the iterate is zero on entry (first red launch); the
@@ -113,18 +119,54 @@ __device__ __forceinline__ T mul_rn(T a, T b)
 }
 
 template <class T>
-__device__ __forceinline__ T relax_cell(T xc, T xl, T xr, T fl, T fr, T fs, T fn, T fb, T ft, T xs,
-                                        T xn, T xb, T xt, T bc, T omega)
+__device__ __forceinline__ void relax_terms(T xc, T xl, T xr, T fl, T fr, T fs, T fn, T fb, T ft, T xs, T xn, T xb,
+                                            T xt, T bc, T &num, T &d)
 {
-    const T d = ((((fl + fr) + fs) + fn) + fb) + ft;
+    d = ((((fl + fr) + fs) + fn) + fb) + ft;
     T f = mul_rn(fl, xl - xc);
     f = fma(fr, xr - xc, f);
     f = fma(fs, xs - xc, f);
     f = fma(fn, xn - xc, f);
     f = fma(fb, xb - xc, f);
     f = fma(ft, xt - xc, f);
-    return relaxable(d) ? fma(omega, relax_div(f - bc, d), xc) : xc;
+    num = f - bc;
 }
+// Two cells from their residuals n and diagonals d (half-sweeps): one branch for
+// the subnormal ones of both.
+template <class T>
+__device__ __forceinline__ void relax_two(T x0, T n0, T d0, T x1, T n1, T d1, T omega, T &v0, T &v1)
+{
+    if constexpr (sizeof(T) == 4) {
+        float q0 = n0 * rcp_ftz(d0), q1 = n1 * rcp_ftz(d1);
+        if (!(d0 >= kTinyDiag && d1 >= kTinyDiag)) {
+            if (!(d0 >= kTinyDiag)) q0 = tiny_quot(n0, d0);
+            if (!(d1 >= kTinyDiag)) q1 = tiny_quot(n1, d1);
+        }
+        v0 = fma(omega, q0, x0);
+        v1 = fma(omega, q1, x1);
+    } else {
+        v0 = d0 > T(0) ? fma(omega, n0 / d0, x0) : x0;
+        v1 = d1 > T(0) ? fma(omega, n1 / d1, x1) : x1;
+    }
+}
+
+// The relaxation of one cell in the one-pass sweeps, whose steps a branch costs
+// their registers and schedule (marching sweep of 512^3: 523 us, 660 with it): the
+// diagonal is scaled by tiny in every cell, 2^24 on a handle with a subnormal face
+// (GridState::tiny) and else 1, and omega holds that factor too.  Powers of 2: the
+// same bits, but for diagonals above 2^102 and changes below 2^-102 on a handle
+// with subnormal faces.  Tried in its place: a second body of the sweep, or a call,
+// for such handles (tables of several grids 5 % slower).
+template <class T>
+__device__ __forceinline__ T relax_cell(T xc, T xl, T xr, T fl, T fr, T fs, T fn, T fb, T ft, T xs,
+                                        T xn, T xb, T xt, T bc, T omega, T tiny)
+{
+    T num, d;
+    relax_terms(xc, xl, xr, fl, fr, fs, fn, fb, ft, xs, xn, xb, xt, bc, num, d);
+    if constexpr (sizeof(T) == 4) return d > 0.f ? fma(omega, num * rcp_ftz(d * tiny), xc) : xc;
+    else return d > T(0) ? fma(omega, num / d, xc) : xc;
+}
+__device__ __forceinline__ float tiny_scale(const GridState *s) { return s->tiny ? kTinyScale : 1.f; }
 
 // The relaxation of FP64 cycles, with the cell's diagonal given by its inverse
 // di = 1 / d (d summed as relax_cell sums it; 0 for a cell without faces),
@@ -274,8 +316,10 @@ __device__ __forceinline__ void half_quad(T *x, const T *b, const T *wx, const T
         v0 = relax_cell_inv(xc0, xl0, xr0, fl0, fr0, fs0, fn0, fb0, ft0, xs0, xn0, xb0, xt0, b0, omega, di0);
         v1 = relax_cell_inv(xc1, xl1, xr1, fl1, fr1, fs1, fn1, fb1, ft1, xs1, xn1, xb1, xt1, b1, omega, di1);
     } else {
-        v0 = relax_cell(xc0, xl0, xr0, fl0, fr0, fs0, fn0, fb0, ft0, xs0, xn0, xb0, xt0, b0, omega);
-        v1 = relax_cell(xc1, xl1, xr1, fl1, fr1, fs1, fn1, fb1, ft1, xs1, xn1, xb1, xt1, b1, omega);
+        T n0, d0, n1, d1;
+        relax_terms(xc0, xl0, xr0, fl0, fr0, fs0, fn0, fb0, ft0, xs0, xn0, xb0, xt0, b0, n0, d0);
+        relax_terms(xc1, xl1, xr1, fl1, fr1, fs1, fn1, fb1, ft1, xs1, xn1, xb1, xt1, b1, n1, d1);
+        relax_two(xc0, n0, d0, xc1, n1, d1, omega, v0, v1);
     }
     Quad<T> out = xq;
     out.v[0] = par ? xq.v[0] : v0;
@@ -462,7 +506,7 @@ __device__ __forceinline__ T zero_start_red(const LevelView &L, int I, int J, in
     d += wz[c];
     if (K + 1 < nz) d += wz[c + sz];
     else if (per & 4) d += wz[c - sz * (nz - 1)];
-    return relaxable(d) ? omega * relax_div(-bc, d) : T(0);
+    return omega * relax_quot(-bc, d);
 }
 
 template <class T>

@@ -122,7 +122,7 @@ __device__ __forceinline__ void item_setup(const TailView &V, int t, int q, cons
     // first cell: faces fx.x (low x), fx.y; second: fx.y, fe
     const float d0 = ((((f.fx.x + f.fx.y) + f.fs.x) + f.fn.x) + f.fb.x) + f.ft.x;
     const float d1 = ((((f.fx.y + f.fe) + f.fs.y) + f.fn.y) + f.fb.y) + f.ft.y;
-    const float i0 = relaxable(d0) ? relax_div(omega, d0) : 0.f, i1 = relaxable(d1) ? relax_div(omega, d1) : 0.f;
+    const float i0 = d0 >= kTinyDiag ? omega * rcp_ftz(d0) : 0.f, i1 = d1 >= kTinyDiag ? omega * rcp_ftz(d1) : 0.f;
     const bool p = s.p;
     o.fo = f.fx.y;
     o.rf = p ? f.fe : f.fx.x;
@@ -151,6 +151,22 @@ __device__ __forceinline__ void item_setup(const TailView &V, int t, int q, cons
     o.side = p ? (unsigned)qe | (unsigned)qw << 16 : (unsigned)qw | (unsigned)qe << 16;
     o.ny = (unsigned)qs | (unsigned)qn << 16;
     o.nz = (unsigned)qb | (unsigned)qt << 16;
+}
+
+// A handle with subnormal faces (GridState::tiny): every face and right-hand side
+// down to the coarsest level is multiplied by 2^24, which leaves the corrections as
+// they are and makes every diagonal, and its inverse, a normal float.  Here the
+// first level's items, after their set-up (scaled as they are loaded, the branch
+// would wait for the loads: 1 us of the launch's 19).
+__device__ __forceinline__ void item_scale(Item &o, float omega)
+{
+    o.fo *= kTinyScale;
+    o.rf *= kTinyScale, o.rs *= kTinyScale, o.rn *= kTinyScale, o.rb *= kTinyScale, o.rt *= kTinyScale;
+    o.bf *= kTinyScale, o.bs *= kTinyScale, o.bn *= kTinyScale, o.bb *= kTinyScale, o.bt *= kTinyScale;
+    const float rd = ((((o.fo + o.rf) + o.rs) + o.rn) + o.rb) + o.rt;
+    const float bd = ((((o.fo + o.bf) + o.bs) + o.bn) + o.bb) + o.bt;
+    o.ri = rd > 0.f ? omega * rcp_ftz(rd) : 0.f;
+    o.bi = bd > 0.f ? omega * rcp_ftz(bd) : 0.f;
 }
 
 __device__ __forceinline__ void item_rhs(int p, float b0, float b1, Item &o)
@@ -340,6 +356,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailView *__rest
     float *sm = (float *)smem_raw;
     __shared__ __align__(16) TailView V;
     __shared__ __align__(8) unsigned long long bar;
+    __shared__ int tiny;  // see item_scale
     const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // the view by one load per thread: read field by field from global memory
     // its cache lines cost a memory latency each, one after the other
@@ -348,6 +365,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailView *__rest
     const bool go = in_cycle(G.st, cyc);
     if (tid < (int)(sizeof(TailView) / 4)) ((unsigned *)&V)[tid] = ((const unsigned *)&G)[tid];
     if (tid == 0) mbar_init(&bar, 1);
+    if (tid == kTailThreads - 1) tiny = G.st->tiny;
     __syncthreads();
     if (!go) return;
     const int nt = V.nt;
@@ -421,6 +439,17 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailView *__rest
         mbar_wait(&bar, 0, kBulkWaitPolls);
         return;
     }
+    if (tiny) {  // the first level's items, the staged right-hand side and faces
+#pragma unroll
+        for (int i = 0; i < kTailItems; i++) item_scale(it0[i], omega);
+        for (int c = tid; c < N0; c += kTailThreads) A0.nat[c] *= kTinyScale;
+        for (int t = 1; t + 1 < nt; t++) {
+            const int N = V.n[t][0] * V.n[t][1] * V.n[t][2];
+            float *w = level_arr(V, t, sm).w;
+            for (int c = tid; c < 3 * N; c += kTailThreads) w[c] *= kTinyScale;
+        }
+        __syncthreads();
+    }
 #pragma unroll
     for (int i = 0; i < kTailItems; i++) {
         const float2 b = *(const float2 *)(A0.nat + 2 * q0[i]);
@@ -479,6 +508,10 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailView *__rest
                 const int row = fdiv(c, V.dx[t]), K = fdiv(row, V.dy[t]);
                 A.b[c] = (double)coarse_rhs(V, t - 1, S, c - row * V.n[t][0], row - K * V.n[t][1], K);
             }
+            __syncthreads();
+        }
+        if (tiny) {
+            for (int c = tid; c < n; c += kTailThreads) A.b[c] *= 1.0 / kTinyScale;
             __syncthreads();
         }
         if (small) {
