@@ -510,7 +510,8 @@ int mg_tune_cache_save(const char *path);
  * shape that does not fit the level, are skipped); *loaded (may be NULL) gets
  * the number of choices read.  MG_ENOTFOUND if the file cannot be opened.
  * When the environment variable MG_TUNE_CACHE names a file, the first tuning
- * of the process loads it and each new choice is appended to it. */
+ * of the process loads it and each new choice is appended to it.  Choices of
+ * the sweep stand where no rule picks the marching sweep (see mg_params.sweep). */
 int mg_tune_cache_load(const char *path, int *loaded);
 
 /* Number of cached choices. */

@@ -264,8 +264,8 @@ int time_sweep(mg_handle *h, int v, float *ms)
     return MG_OK;
 }
 
-// Sweeps: MG_SWEEP_HALF, a forced one-pass shape, a cached choice, the marching
-// sweep where its rule picks it, or the fastest of the half-sweep pair and every
+// Sweeps: MG_SWEEP_HALF, a forced one-pass shape, the marching sweep where its
+// rule picks it, a cached choice, or the fastest of the half-sweep pair and every
 // whole-row shape that fits (cached like the launch shapes).
 int tune_sweep(mg_handle *h)
 {
@@ -285,6 +285,18 @@ int tune_sweep(mg_handle *h)
         choose((forced > 0 && sweep_fits(n, h->per, forced, h->mixed)) ? forced : 0);
         return MG_OK;
     }
+    // the marching sweep by rule, in chunks of its own (reported as the shape
+    // whose chunks hold them); where it is not the faster one, a cached choice, or
+    // the half-sweep pair against the whole-row shapes, timed.  The rule comes first:
+    // a file of choices may have been timed before the marching sweep was there
+    const int kc = h->mixed ? march_chunk(n, h->per) : 0;
+    if (kc) {
+        h->mkc[0] = kc;
+        int v = kMarchVariant;
+        while (v + 1 < kSweepVariants && sweep_shape(v).Kc < kc) v++;
+        h->tile[MG_TILE_SWEEP][0] = (signed char)v;
+        return MG_OK;
+    }
     TuneKey key;
     memset(&key, 0, sizeof(key));
     key.kind = MG_TILE_SWEEP;
@@ -299,17 +311,6 @@ int tune_sweep(mg_handle *h)
             choose(it->second);
             return MG_OK;
         }
-    }
-    // the marching sweep by rule, in chunks of its own (reported as the shape
-    // whose chunks hold them); where it is not the faster one, the half-sweep
-    // pair against the whole-row shapes, timed
-    const int kc = h->mixed ? march_chunk(n, h->per) : 0;
-    if (kc) {
-        h->mkc[0] = kc;
-        int v = kMarchVariant;
-        while (v + 1 < kSweepVariants && sweep_shape(v).Kc < kc) v++;
-        h->tile[MG_TILE_SWEEP][0] = (signed char)v;
-        return MG_OK;
     }
     float t[kSweepVariants];
     for (int v = 0; v < kSweepVariants; v++) t[v] = -1.f;

@@ -1,0 +1,36 @@
+"""The finest level's sweep: the marching sweep's rule stands before a saved
+choice (files of an earlier version hold choices timed against other kernels),
+and the choice that a handle reports can be run on its level."""
+import pytest
+
+from paper_1410_8568_gb300 import gbmg
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def solver(shape, bc):
+    g = torch.Generator(device="cuda").manual_seed(sum(shape))
+    rho = torch.exp(torch.rand(shape[::-1], dtype=torch.float64, device="cuda", generator=g))
+    return gbmg.Solver(shape, bc, rho=rho)
+
+
+@pytest.mark.parametrize("saved", [0, 1, 7])
+def test_a_saved_choice_does_not_replace_the_rule(tmp_path, saved):
+    shape, bc = (128, 128, 128), (1, 1, 0)
+    gbmg.tune_cache_clear()
+    with solver(shape, bc) as S:
+        rule = S.tile_choice(gbmg.TILE_SWEEP, 0)
+    assert gbmg.sweep_shape(rule)[2] > 0  # it marches
+    src = tmp_path / "tune.txt"
+    src.write_text("3 1 3 128 128 128 %d\n" % saved)
+    gbmg.tune_cache_clear()
+    assert gbmg.tune_cache_load(str(src)) == 1
+    with solver(shape, bc) as S:
+        assert S.tile_choice(gbmg.TILE_SWEEP, 0) == rule
+        # below the march's sizes the saved choice is taken
+    src.write_text("3 1 3 64 64 64 3\n")
+    assert gbmg.tune_cache_load(str(src)) == 1
+    with solver((64, 64, 64), bc) as S:
+        assert S.tile_choice(gbmg.TILE_SWEEP, 0) == 3
+    gbmg.tune_cache_clear()
