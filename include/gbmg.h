@@ -367,8 +367,9 @@ int mg_restrict_residual(mg_handle *h, int level, int prec, const void *b, const
  * choice on that level.  MG_EINVAL if the shape does not fit the level: an
  * even number of cells along a periodic y or z axis, and for a whole-row shape
  * rows of a multiple of 4 cells, at most a third of the shape's threads quads
- * per row; for a tiled shape rows of a multiple of its tile_x cells and
- * prec = MG_PREC_MIXED. */
+ * per row; for a tiled shape prec = MG_PREC_MIXED and rows of a multiple of its
+ * tile_x cells or the shape that the handle reports as its choice for the level
+ * (mg_tile_choice). */
 int mg_smooth_onepass(mg_handle *h, int level, int prec, const void *b, void *x, void *work, int sweeps,
                       int variant);
 

@@ -1701,9 +1701,12 @@ int mg_smooth_onepass(mg_handle *h, int level, int prec, const void *b, void *x,
     if (prec != MG_PREC_FP64 && prec != MG_PREC_MIXED) return MG_EINVAL;
     if (prec == MG_PREC_MIXED && !h->mixed) return MG_EINVAL;
     const HLevel &L = h->lev[level];
-    // the handle's choice on the finest level (a marching sweep by its own chunk)
-    const bool own = variant == 0 && level == 0;
-    if (own) variant = h->tile[MG_TILE_SWEEP][0];
+    // the handle's choice on the finest level (a marching sweep by its own chunk),
+    // asked for as 0 or, where the shape reported does not fit the rows, by its number
+    const int choice = h->tile[MG_TILE_SWEEP][0];
+    const bool fits = sweep_fits(L.n, h->per, variant, prec == MG_PREC_MIXED);
+    const bool own = level == 0 && (variant == 0 || (variant == choice && !fits));
+    if (variant == 0 && level == 0) variant = choice;
     const int kc = own && prec == MG_PREC_MIXED ? h->mkc[0] : 0;
     if (!kc && !sweep_fits(L.n, h->per, variant, prec == MG_PREC_MIXED)) return MG_EINVAL;
     LevelView v;

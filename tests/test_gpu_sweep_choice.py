@@ -34,3 +34,18 @@ def test_a_saved_choice_does_not_replace_the_rule(tmp_path, saved):
     with solver((64, 64, 64), bc) as S:
         assert S.tile_choice(gbmg.TILE_SWEEP, 0) == 3
     gbmg.tune_cache_clear()
+
+
+@pytest.mark.parametrize("shape,bc", [((192, 160, 128), (1, 1, 0)), ((320, 128, 96), (0, 1, 0))])
+def test_the_reported_choice_runs_on_its_level(shape, bc):
+    gbmg.tune_cache_clear()
+    with solver(shape, bc) as S:
+        choice = S.tile_choice(gbmg.TILE_SWEEP, 0)
+        assert gbmg.sweep_shape(choice)[2] > 0
+        g = torch.Generator(device="cuda").manual_seed(7)
+        x = torch.randn(shape[::-1], dtype=torch.float32, device="cuda", generator=g)
+        b = torch.randn(shape[::-1], dtype=torch.float32, device="cuda", generator=g)
+        want, work = x.clone(), torch.zeros_like(x)
+        S.smooth(0, b, want, 2, prec=gbmg.MIXED)
+        S.smooth_onepass(0, b, x, work, 2, prec=gbmg.MIXED, variant=choice)
+        assert torch.equal(x, want)
