@@ -125,6 +125,21 @@ def kernel_source_hash():
     return h.hexdigest()[:16]
 
 
+def finest_kernel(sv, v0):
+    """The kernel of the finest level's relaxation: one-pass sweep shape sv (0: half-sweeps of tile shape v0)."""
+    from paper_1410_8568_gb300 import gbmg
+    if sv == 0:
+        return ("FP32 half-sweep of level 0 (one red or black colour), launch shape %d (%d threads x %d quads)" %
+                ((v0,) + gbmg.tile_shape(v0)))
+    threads, planes, tile_x = gbmg.sweep_shape(sv)
+    if tile_x:
+        # the blocks have 16 row warps; the shape's thread count includes a warp whose work they share
+        return ("FP32 marching red-black sweep of level 0 (both colours in one launch, k_march): 512 threads, tiles "
+                "of up to %d cells along x and 14 rows, up to %d planes per block" % (tile_x, planes))
+    return ("FP32 one-pass red-black sweep of level 0 (both colours in one launch), shape %d (%d threads, whole rows, "
+            "%d planes per block)" % (sv, threads, planes))
+
+
 def profiled_traffic(workload, kernel="smooth"):
     """DRAM bytes per launch of the dominant kernel (the finest-level half-sweep,
     "smooth", or one-pass sweep, "sweep") from the committed ncu summary, or None
@@ -618,10 +633,10 @@ ACT_BPC = {"half": 20.0, "sweep": 24.0}
 # the old iterate, b and the 3 face arrays once and writes the new iterate: the
 # algorithmic bytes (its halo rows and planes are re-read through L2).
 # FP64 residual of a refinement step: reads p, b - mean b and 3 FP64 faces,
-# writes the FP32 residual (44 B); 6 differences, 1 product and 5 fused
-# multiply-adds, the subtraction from b and the scale (14 FP64 operations) and
-# the FP64 -> FP32 conversion, which this GPU also issues to its FP64 pipe.
-RES_BPC, RES_FP64_OPS = 44.0, 15.0
+# writes the FP32 residual (44 B); per pair of cells 9 differences (the z faces
+# and the x face inside the pair serve both their cells) and 12 fused
+# multiply-adds, the scale and the conversion to FP32 on the bits.
+RES_BPC, RES_FP64_OPS = 44.0, 10.5
 
 
 def oracle_reference_run(P, tol=TOL):
@@ -872,12 +887,7 @@ def run_single(args, rank, world, local_rank, dist):
                     "h2d_bytes_per_step": 3 * 8 * N, "d2h_bytes_per_step": 8 * N},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": ("FP32 one-pass red-black sweep of level 0 (both colours in one launch), "
-                                    "shape %d (%d threads, %d planes per block, tile of %d cells along x; "
-                                    "0: whole rows)" % ((sv,) + gbmg.sweep_shape(sv)))
-                                   if sv > 0 else
-                                   ("FP32 half-sweep of level 0 (one red or black colour), launch shape %d "
-                                    "(%d threads x %d quads)" % ((v0,) + gbmg.tile_shape(v0))),
+                         "kernel": finest_kernel(sv, v0),
                          "bytes_rule": "algorithmic: 6 s = 24 B per cell per full red+black sweep (%s)" %
                                        ("one launch" if sv > 0 else "half per colour launch: 12 B x cells"),
                          "bytes_per_launch": bytes_launch,
