@@ -291,7 +291,7 @@ bool sweep_fits(const int n[3], int per, int v, bool fp32)
 {
     if (v < 1 || v >= kSweepVariants) return false;
     const SweepShape sh = sweep_shape(v);
-    if (sh.tile_x) return fp32 && staged_fits(n, per);
+    if (sh.tile_x) return fp32 && tiled_fits(n, per);
     // rows of whole quads, at least one own row per strip, and an even number
     // of cells along every periodic axis (else the colours do not alternate
     // across the wrap)

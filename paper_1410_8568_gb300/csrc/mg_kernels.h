@@ -131,9 +131,9 @@ template <class T> void launch_sweep(const Table &, int dir, double omega, int f
                                      cudaStream_t);
 // the marching one-pass sweep of FP32 cycles (mg_march.cu) on levels with rows of
 // whole quads: march_chunk gives the planes per block (0: half-sweeps are
-// faster); staged_fits: the levels the public shapes 7 .. 10 are offered for
+// faster); tiled_fits: the levels the public shapes 7 .. 10 are offered for
 bool march_fits(const int n[3], int per);
-bool staged_fits(const int n[3], int per);
+bool tiled_fits(const int n[3], int per);
 int march_chunk(const int n[3], int per);
 int march_layout(LevelView &v, int kc);
 void launch_march(const Table &, int dir, double omega, int flags, const OuterView *ov, cudaStream_t);

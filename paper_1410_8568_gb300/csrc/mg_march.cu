@@ -487,7 +487,7 @@ bool march_fits(const int n[3], int per)
     return (n[0] & 3) == 0 && n[1] >= 2 && n[2] >= 2 && !((per & 2) && (n[1] & 1)) && !((per & 4) && (n[2] & 1));
 }
 
-bool staged_fits(const int n[3], int per) { return n[0] % 128 == 0 && march_fits(n, per); }
+bool tiled_fits(const int n[3], int per) { return n[0] % 128 == 0 && march_fits(n, per); }
 
 // tiles of a plane: strips of rows x tiles of quads
 static int march_tiles(const int n[3], int *strips)
