@@ -369,7 +369,8 @@ int mg_restrict_residual(mg_handle *h, int level, int prec, const void *b, const
  * rows of a multiple of 4 cells, at most a third of the shape's threads quads
  * per row; for a tiled shape prec = MG_PREC_MIXED and rows of a multiple of its
  * tile_x cells or the shape that the handle reports as its choice for the level
- * (mg_tile_choice). */
+ * (mg_tile_choice).  x and work are 16-byte aligned, and for a tiled shape b too
+ * (MG_EINVAL). */
 int mg_smooth_onepass(mg_handle *h, int level, int prec, const void *b, void *x, void *work, int sweeps,
                       int variant);
 

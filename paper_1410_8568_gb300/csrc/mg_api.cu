@@ -1707,8 +1707,18 @@ int mg_smooth_onepass(mg_handle *h, int level, int prec, const void *b, void *x,
     const bool fits = sweep_fits(L.n, h->per, variant, prec == MG_PREC_MIXED);
     const bool own = level == 0 && (variant == 0 || (variant == choice && !fits));
     if (variant == 0 && level == 0) variant = choice;
-    const int kc = own && prec == MG_PREC_MIXED ? h->mkc[0] : 0;
+    int kc = own && prec == MG_PREC_MIXED ? h->mkc[0] : 0;
     if (!kc && !sweep_fits(L.n, h->per, variant, prec == MG_PREC_MIXED)) return MG_EINVAL;
+    // the marching sweep copies 16 bytes at a time, of b too (the whole-row shapes
+    // read that by single values): a whole-row shape takes the place of the handle's
+    // choice for such a b, a marching shape asked for by its number is refused
+    if ((kc || variant >= kMarchVariant) && (((uintptr_t)b | (uintptr_t)x | (uintptr_t)work) & 15) != 0) {
+        kc = 0;
+        int v = own && (((uintptr_t)x | (uintptr_t)work) & 15) == 0 ? 1 : kMarchVariant;
+        while (v < kMarchVariant && !sweep_fits(L.n, h->per, v, true)) v++;
+        if (v == kMarchVariant) return MG_EINVAL;
+        variant = v;
+    }
     LevelView v;
     memset(&v, 0, sizeof(v));
     for (int d = 0; d < 3; d++) {

@@ -49,3 +49,27 @@ def test_the_reported_choice_runs_on_its_level(shape, bc):
         S.smooth(0, b, want, 2, prec=gbmg.MIXED)
         S.smooth_onepass(0, b, x, work, 2, prec=gbmg.MIXED, variant=choice)
         assert torch.equal(x, want)
+
+
+def test_a_right_hand_side_at_an_odd_element():
+    """The marching sweep copies quads of b: an unaligned one is refused by number, and
+    the handle's choice runs a whole-row shape on it."""
+    shape, bc = (192, 160, 128), (1, 1, 0)
+    with solver(shape, bc) as S:
+        g = torch.Generator(device="cuda").manual_seed(8)
+        x = torch.randn(shape[::-1], dtype=torch.float32, device="cuda", generator=g)
+        b = torch.empty(x.numel() + 1, dtype=torch.float32, device="cuda")[1:].view(x.shape)
+        b.copy_(torch.randn(shape[::-1], dtype=torch.float32, device="cuda", generator=g))
+        assert b.data_ptr() % 16 == 4
+        want, work = x.clone(), torch.zeros_like(x)
+        S.smooth(0, b, want, 2, prec=gbmg.MIXED)
+        S.smooth_onepass(0, b, x, work, 2, prec=gbmg.MIXED, variant=0)
+        assert torch.equal(x, want)
+    shape = (256, 32, 16)
+    with solver(shape, bc) as S:
+        x = torch.zeros(shape[::-1], dtype=torch.float32, device="cuda")
+        b = torch.zeros(x.numel() + 1, dtype=torch.float32, device="cuda")[1:].view(x.shape)
+        for v in (7, 10):
+            with pytest.raises(gbmg.MGError) as e:
+                S.smooth_onepass(0, b, x, x.clone(), 1, prec=gbmg.MIXED, variant=v)
+            assert e.value.code == gbmg.EINVAL
